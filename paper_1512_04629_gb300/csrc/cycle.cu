@@ -106,12 +106,22 @@ template <> struct Vec<__nv_bfloat16> {
     }
 };
 
-// sum over one CSR row by a group of T lanes (all lanes get the sum)
-template <typename VT, typename XT, int T, class G>
+// acc + a x, or acc - a x (SUB): one fused multiply-add either way.  The
+// residuals b - sum a x start their accumulator at b, so the subtraction of
+// the finished sum is not an operation of its own -- on this part an FP64
+// warp instruction holds its pipe for 16 clocks, and a 7-entry row's residual
+// is then 7 of them instead of 8.
+template <bool SUB, typename XT> __device__ __forceinline__ XT mac(XT acc, XT a, XT x) {
+    return SUB ? acc - a * x : acc + a * x;
+}
+
+// init + sum (SUB: init - sum) over one CSR row by a group of T lanes (all
+// lanes get the result; init is the group's first lane's)
+template <typename VT, typename XT, int T, bool SUB = false, class G>
 __device__ __forceinline__ XT csr_row_sum(int32_t p0, int32_t p1, int t, const int32_t *__restrict__ ci,
-                                          const VT *__restrict__ v, G gather) {
+                                          const VT *__restrict__ v, G gather, XT init = XT(0)) {
     constexpr int V = Vec<VT>::V;
-    XT acc = XT(0);
+    XT acc = t == 0 ? init : XT(0);
     for (int32_t q = (p0 & ~(V - 1)) + t * V; q < p1; q += T * V) {
         VT vv[V];
         int32_t cc[V];
@@ -119,7 +129,7 @@ __device__ __forceinline__ XT csr_row_sum(int32_t p0, int32_t p1, int t, const i
 #pragma unroll
         for (int u = 0; u < V; ++u) {
             int32_t e = q + u;
-            if (e >= p0 && e < p1) acc += cvt<VT, XT>(vv[u]) * gather(cc[u]);
+            if (e >= p0 && e < p1) acc = mac<SUB>(acc, cvt<VT, XT>(vv[u]), gather(cc[u]));
         }
     }
 #pragma unroll
@@ -155,8 +165,8 @@ constexpr int kShortMax = 8;  // widest slice of the load-first path
 // a slice of width W (W <= 8): every value and column load first, then every
 // gather, then the products in k order -- short rows (interpolation P,
 // coarse operators) otherwise pay a load -> gather round trip per entry
-template <int W, typename VT, typename XT, bool D16, class G, bool CS = false>
-__device__ __forceinline__ XT sell_short_sum(int32_t off, int32_t row, const SellIdx &ix,
+template <int W, typename VT, typename XT, bool D16, bool CS, bool SUB, class G>
+__device__ __forceinline__ XT sell_short_sum(XT acc, int32_t off, int32_t row, const SellIdx &ix,
                                              const VT *__restrict__ sv, G gather) {
     VT v[W];
     int32_t c[W];
@@ -168,64 +178,73 @@ __device__ __forceinline__ XT sell_short_sum(int32_t off, int32_t row, const Sel
     XT g[W];
 #pragma unroll
     for (int k = 0; k < W; ++k) g[k] = gather(c[k]);
-    XT acc = XT(0);
 #pragma unroll
-    for (int k = 0; k < W; ++k) acc += cvt<VT, XT>(v[k]) * g[k];
+    for (int k = 0; k < W; ++k) acc = mac<SUB>(acc, cvt<VT, XT>(v[k]), g[k]);
     return acc;
 }
 
-// the same for the last W (< 4) entries of a lane in the SELL-C kernels,
-// added into acc in k order after every load and gather is in flight
-template <int W, typename VT, typename XT, bool D16, bool CS, class G>
-__device__ __forceinline__ void sell_tail_acc(XT &acc, int32_t off, int32_t row, const SellIdx &ix,
-                                              const VT *__restrict__ sv, G gather) {
-    VT v[W];
-    int32_t c[W];
-#pragma unroll
-    for (int k = 0; k < W; ++k) {
-        v[k] = ld_ro<CS>(sv + off + k * 32);
-        c[k] = sell_col<D16, CS>(ix, off + k * 32, row);
+// the same for a width known at run time (1..8; the same for the whole warp)
+template <typename VT, typename XT, bool D16, bool CS, bool SUB, class G>
+__device__ __forceinline__ XT sell_short_any(XT acc, int32_t w, int32_t off, int32_t row, const SellIdx &ix,
+                                             const VT *__restrict__ sv, G gather) {
+    switch (w) {
+        case 1: return sell_short_sum<1, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 2: return sell_short_sum<2, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 3: return sell_short_sum<3, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 4: return sell_short_sum<4, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 5: return sell_short_sum<5, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 6: return sell_short_sum<6, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 7: return sell_short_sum<7, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        case 8: return sell_short_sum<8, VT, XT, D16, CS, SUB>(acc, off, row, ix, sv, gather);
+        default: return acc;
     }
-    XT g[W];
-#pragma unroll
-    for (int k = 0; k < W; ++k) g[k] = gather(c[k]);
-#pragma unroll
-    for (int k = 0; k < W; ++k) acc += cvt<VT, XT>(v[k]) * g[k];
 }
 
-// sum over the row stored at SELL position pos (slice pos / 32, lane pos % 32),
-// entries in k order whatever the path; SHORT: slices of width <= 8 take the
-// load-everything-first path (the transfer operators P and R, whose rows are
-// short; the relaxation kernels measured slower with it)
-template <typename VT, typename XT, bool D16, bool SHORT = false, bool CS = false, class G>
+// init + sum (SUB: init - sum) over the row stored at SELL position pos
+// (slice pos / 32, lane pos % 32), entries in k order whatever the path;
+// SHORT: slices of width <= 8 take the load-everything-first path (the
+// transfer operators P and R, whose rows are short; the relaxation kernels
+// measured slower with it)
+template <typename VT, typename XT, bool D16, bool SHORT, bool CS, bool SUB, class G>
 __device__ __forceinline__ XT sell_row_sum(int32_t pos, int32_t row, const int32_t *__restrict__ soff,
                                            const int32_t *__restrict__ sw, const SellIdx &ix,
-                                           const VT *__restrict__ sv, G gather) {
+                                           const VT *__restrict__ sv, G gather, XT init = XT(0)) {
     int32_t s = pos >> 5, lane = pos & 31;
     int32_t off = __ldg(soff + s) + lane, w = __ldg(sw + s);
-    if constexpr (SHORT) {
-        switch (w) {  // uniform over the warp (one slice)
-            case 1: return sell_short_sum<1, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 2: return sell_short_sum<2, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 3: return sell_short_sum<3, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 4: return sell_short_sum<4, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 5: return sell_short_sum<5, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 6: return sell_short_sum<6, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 7: return sell_short_sum<7, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            case 8: return sell_short_sum<8, VT, XT, D16, G, CS>(off, row, ix, sv, gather);
-            default: break;
-        }
+    if constexpr (SHORT) {  // w: uniform over the warp (one slice)
+        if (w <= kShortMax) return sell_short_any<VT, XT, D16, CS, SUB>(init, w, off, row, ix, sv, gather);
     }
-    XT acc = XT(0);
+    XT acc = init;
 #pragma unroll 4
     for (int32_t k = 0; k < w; ++k) {
         int32_t p = off + k * 32;
-        acc += cvt<VT, XT>(ld_ro<CS>(sv + p)) * gather(sell_col<D16, CS>(ix, p, row));
+        acc = mac<SUB>(acc, cvt<VT, XT>(ld_ro<CS>(sv + p)), gather(sell_col<D16, CS>(ix, p, row)));
     }
     return acc;
 }
 
-enum Op { kPre = 0, kPost = 1, kSpmv = 2, kSpmvAdd = 3, kSpmvScale = 4, kResX = 5 };
+enum Op { kPost = 1, kSpmv = 2, kSpmvAdd = 3, kSpmvScale = 4, kResX = 5 };
+
+// the operations that form b - A x: their row accumulators start at b
+template <int OP> constexpr bool kIsResid = OP == kPost || OP == kResX;
+
+// what an operation does with its row's sum s (b - A x for the residual forms)
+template <typename XT, int OP>
+__device__ __forceinline__ void row_store(int32_t i, XT s, const XT *__restrict__ dinv, const XT *__restrict__ x,
+                                          XT *__restrict__ o1, XT *__restrict__ o2) {
+    if (OP == kPost) {
+        o1[i] = x[i] + dinv[i] * s;
+    } else if (OP == kSpmv) {
+        o1[i] = s;
+    } else if (OP == kSpmvScale) {
+        o1[i] = s;
+        o2[i] = s * dinv[i];
+    } else if (OP == kResX) {
+        o2[i] = s;
+    } else {
+        o1[i] += s;
+    }
+}
 
 template <typename VT, typename XT, int T, int OP>
 __global__ void __launch_bounds__(kThreads)
@@ -238,26 +257,10 @@ csr_op_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restri
     int t = (int)(g % T);
     int32_t p0 = 0, p1 = 0;
     if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
-    XT s;
-    if (OP == kPre) s = csr_row_sum<VT, XT, T>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(b + j) * __ldg(dinv + j); });
-    else s = csr_row_sum<VT, XT, T>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); });
+    const XT init = kIsResid<OP> && i < n && t == 0 ? b[i] : XT(0);
+    const XT s = csr_row_sum<VT, XT, T, kIsResid<OP>>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); }, init);
     if (i >= n || t != 0) return;
-    if (OP == kPre) {
-        XT bi = b[i];
-        o1[i] = bi * dinv[i];
-        o2[i] = bi - s;
-    } else if (OP == kPost) {
-        o1[i] = x[i] + dinv[i] * (b[i] - s);
-    } else if (OP == kSpmv) {
-        o1[i] = s;
-    } else if (OP == kSpmvScale) {
-        o1[i] = s;
-        o2[i] = s * dinv[i];
-    } else if (OP == kResX) {
-        o2[i] = b[i] - s;
-    } else {
-        o1[i] += s;
-    }
+    row_store<XT, OP>(i, s, dinv, x, o1, o2);
 }
 
 // One lane per row of a SELL-32 operator; SHORT: every slice fits the
@@ -278,24 +281,15 @@ sell_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
     XT own = XT(0);
     if (OP == kSpmvAdd) own = o1[i];
     if (OP == kSpmvScale) own = dinv[i];
-    XT s;
-    if (OP == kPre) s = sell_row_sum<VT, XT, D16, SHORT || kTransfer, CS>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(b + j) * __ldg(dinv + j); });
-    else s = sell_row_sum<VT, XT, D16, SHORT || kTransfer, CS>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(x + j); });
-    if (OP == kPre) {
-        XT bi = b[i];
-        o1[i] = bi * dinv[i];
-        o2[i] = bi - s;
-    } else if (OP == kPost) {
-        o1[i] = x[i] + dinv[i] * (b[i] - s);
-    } else if (OP == kSpmv) {
-        o1[i] = s;
-    } else if (OP == kSpmvScale) {
+    const XT init = kIsResid<OP> ? b[i] : XT(0);
+    const XT s = sell_row_sum<VT, XT, D16, SHORT || kTransfer, CS, kIsResid<OP>>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(x + j); }, init);
+    if (OP == kSpmvScale) {
         o1[i] = s;
         o2[i] = s * own;
-    } else if (OP == kResX) {
-        o2[i] = b[i] - s;
-    } else {
+    } else if (OP == kSpmvAdd) {
         o1[i] = own + s;
+    } else {
+        row_store<XT, OP>(i, s, dinv, x, o1, o2);
     }
 }
 
@@ -308,12 +302,11 @@ sell_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
 // unpartitioned kernels', so the results are the same bits.
 // ---------------------------------------------------------------------------
 __global__ void part_exchange_kernel(int64_t nghost, const int32_t *__restrict__ gcol, const double *__restrict__ src,
-                                     const double *__restrict__ scale, double *__restrict__ gbuf) {
+                                     double *__restrict__ gbuf) {
     pdl_begin();
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nghost) return;
-    const int32_t j = __ldg(gcol + k);
-    gbuf[k] = scale ? __ldg(src + j) * __ldg(scale + j) : __ldg(src + j);
+    gbuf[k] = __ldg(src + __ldg(gcol + k));
 }
 
 // block of row i (rows past the end, which gather nothing, get block 0)
@@ -323,17 +316,17 @@ __device__ __forceinline__ int part_of(const PartView &pv, int32_t i) {
     return p;
 }
 
-// where row i's gathers read: owned columns from src + col0[p] (times
-// scale + col0[p] when given), ghosts from gbuf + goff[p]
+// where row i's gathers read: owned columns from src + col0[p], ghosts from
+// gbuf + goff[p]
 struct PartRow {
-    const double *xl, *dl, *g;
+    const double *xl, *g;
     int32_t nloc;
+    __device__ __forceinline__ double operator()(int32_t c) const { return c < nloc ? __ldg(xl + c) : __ldg(g + (c - nloc)); }
 };
-__device__ __forceinline__ PartRow part_row(const PartView &pv, int32_t i, int32_t n, const double *src,
-                                            const double *scale) {
+__device__ __forceinline__ PartRow part_row(const PartView &pv, int32_t i, int32_t n, const double *src) {
     const int p = i < n ? part_of(pv, i) : 0;
     const int32_t c0 = __ldg(pv.col0 + p);
-    return PartRow{src + c0, scale ? scale + c0 : nullptr, pv.gbuf + __ldg(pv.goff + p), __ldg(pv.col0 + p + 1) - c0};
+    return PartRow{src + c0, pv.gbuf + __ldg(pv.goff + p), __ldg(pv.col0 + p + 1) - c0};
 }
 
 template <int T, int OP>
@@ -347,49 +340,23 @@ part_op_kernel(int32_t n, const int32_t *__restrict__ rp, PartView pv, const dou
     int t = (int)(g % T);
     int32_t p0 = 0, p1 = 0;
     if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
-    double s;
-    if (OP == kPre) {
-        const PartRow pr = part_row(pv, i, n, b, dinv);
-        s = csr_row_sum<double, double, T>(p0, p1, t, pv.cext, v, [&](int32_t c) {
-            return c < pr.nloc ? __ldg(pr.xl + c) * __ldg(pr.dl + c) : __ldg(pr.g + (c - pr.nloc));
-        });
-    } else {
-        const PartRow pr = part_row(pv, i, n, x, nullptr);
-        s = csr_row_sum<double, double, T>(p0, p1, t, pv.cext, v, [&](int32_t c) {
-            return c < pr.nloc ? __ldg(pr.xl + c) : __ldg(pr.g + (c - pr.nloc));
-        });
-    }
+    const double init = kIsResid<OP> && i < n && t == 0 ? b[i] : 0.0;
+    const double s = csr_row_sum<double, double, T, kIsResid<OP>>(p0, p1, t, pv.cext, v, part_row(pv, i, n, x), init);
     if (i >= n || t != 0) return;
-    if (OP == kPre) {
-        double bi = b[i];
-        o1[i] = bi * dinv[i];
-        o2[i] = bi - s;
-    } else if (OP == kPost) {
-        o1[i] = x[i] + dinv[i] * (b[i] - s);
-    } else if (OP == kSpmv) {
-        o1[i] = s;
-    } else if (OP == kSpmvScale) {
-        o1[i] = s;
-        o2[i] = s * dinv[i];
-    } else if (OP == kResX) {
-        o2[i] = b[i] - s;
-    } else {
-        o1[i] += s;
-    }
+    row_store<double, OP>(i, s, dinv, x, o1, o2);
 }
 
-// the exchange for an operator whose products gather src (times scale)
-void part_exchange(const PartView &pv, const double *src, const double *scale, cudaStream_t s) {
+// the exchange for an operator whose products gather src
+void part_exchange(const PartView &pv, const double *src, cudaStream_t s) {
     if (pv.nghost == 0) return;
-    { pdl_launch(part_exchange_kernel, (int)div_up(pv.nghost, (int64_t)kThreads), kThreads, 0, s, pv.nghost, pv.gcol, src, scale, pv.gbuf); ::amg::count_launch(); }
+    { pdl_launch(part_exchange_kernel, (int)div_up(pv.nghost, (int64_t)kThreads), kThreads, 0, s, pv.nghost, pv.gcol, src, pv.gbuf); ::amg::count_launch(); }
 }
 
 template <int OP>
 void part_op(const CycMat<double> &A, const double *b, const double *dinv, const double *x, double *o1, double *o2,
              cudaStream_t s) {
     const int32_t n = A.nrows;
-    if (OP == kPre) part_exchange(A.part, b, dinv, s);
-    else part_exchange(A.part, x, nullptr, s);
+    part_exchange(A.part, x, s);
     // one lane per row: the order of the unpartitioned one-lane kernels
     { pdl_launch(part_op_kernel<1, OP>, (int)div_up((int64_t)n, (int64_t)kThreads), kThreads, 0, s, n, A.rp, A.part, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
@@ -416,74 +383,33 @@ sell_lanes_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t 
     const bool valid = pos < n;
     const int32_t i = valid ? (perm ? __ldg(perm + pos) : pos) : 0;
     const int32_t off = __ldg(soff + slice) + lane, w = __ldg(sw + slice);
-    auto gather = [&](int32_t j) {
-        if (OP == kPre) return __ldg(b + j) * __ldg(dinv + j);
-        return __ldg(x + j);
-    };
+    auto gather = [&](int32_t j) { return __ldg(x + j); };
+    constexpr bool SUB = kIsResid<OP>;
     XT acc = XT(0);
     if (valid) {
+        if (SUB && t == 0) acc = b[i];
         const int32_t nk = w / T;  // entries of this lane
         int32_t k = 0;
         if ((OP == kSpmvAdd || OP == kSpmvScale) && nk <= kShortMax) {
             // transfers: a lane's part of a row is short, so all of it loads
             // first (nk is the same for the whole warp), rather than one
             // load -> gather round trip per entry in the tail loop
-            switch (nk) {
-                case 1: acc = sell_short_sum<1, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 2: acc = sell_short_sum<2, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 3: acc = sell_short_sum<3, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 4: acc = sell_short_sum<4, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 5: acc = sell_short_sum<5, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 6: acc = sell_short_sum<6, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 7: acc = sell_short_sum<7, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                case 8: acc = sell_short_sum<8, VT, XT, D16, decltype(gather), CS>(off, i, ix, sv, gather); break;
-                default: break;
-            }
+            acc = sell_short_any<VT, XT, D16, CS, SUB>(acc, nk, off, i, ix, sv, gather);
             k = nk;
         }
-        for (; k + U <= nk; k += U) {
-            VT v[U];
-            int32_t c[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int32_t p = off + (k + u) * 32;
-                v[u] = ld_ro<CS>(sv + p);
-                c[u] = sell_col<D16, CS>(ix, p, i);
-            }
-            XT g[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) g[u] = gather(c[u]);
-#pragma unroll
-            for (int u = 0; u < U; ++u) acc += cvt<VT, XT>(v[u]) * g[u];
-        }
+        for (; k + U <= nk; k += U) acc = sell_short_sum<U, VT, XT, D16, CS, SUB>(acc, off + k * 32, i, ix, sv, gather);
         // the last nk - k < U entries, loaded together (a warp-uniform count)
         switch (nk - k) {
-            case 1: sell_tail_acc<1, VT, XT, D16, CS>(acc, off + k * 32, i, ix, sv, gather); break;
-            case 2: sell_tail_acc<2, VT, XT, D16, CS>(acc, off + k * 32, i, ix, sv, gather); break;
-            case 3: sell_tail_acc<3, VT, XT, D16, CS>(acc, off + k * 32, i, ix, sv, gather); break;
+            case 1: acc = sell_short_sum<1, VT, XT, D16, CS, SUB>(acc, off + k * 32, i, ix, sv, gather); break;
+            case 2: acc = sell_short_sum<2, VT, XT, D16, CS, SUB>(acc, off + k * 32, i, ix, sv, gather); break;
+            case 3: acc = sell_short_sum<3, VT, XT, D16, CS, SUB>(acc, off + k * 32, i, ix, sv, gather); break;
             default: break;
         }
     }
 #pragma unroll
     for (int o = 16; o >= C; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (!valid || t != 0) return;
-    const XT sum = acc;
-    if (OP == kPre) {
-        XT bi = b[i];
-        o1[i] = bi * dinv[i];
-        o2[i] = bi - sum;
-    } else if (OP == kPost) {
-        o1[i] = x[i] + dinv[i] * (b[i] - sum);
-    } else if (OP == kSpmv) {
-        o1[i] = sum;
-    } else if (OP == kSpmvScale) {
-        o1[i] = sum;
-        o2[i] = sum * dinv[i];
-    } else if (OP == kResX) {
-        o2[i] = b[i] - sum;
-    } else {
-        o1[i] += sum;
-    }
+    row_store<XT, OP>(i, acc, dinv, x, o1, o2);
 }
 
 template <typename VT, typename XT, int OP, int C>
@@ -566,36 +492,18 @@ void dispatch_op(const CycMat<VT> &A, const XT *b, const XT *dinv, const XT *x, 
 // ---------------------------------------------------------------------------
 // deterministic block reduction with last-block finish
 // ---------------------------------------------------------------------------
-template <int NV>
-__device__ __forceinline__ void block_reduce(double (&v)[NV]) {
-    __shared__ double sh[NV][kThreads / 32];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double x = v[k];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) sh[k][w] = x;
-    }
-    __syncthreads();
-    if (w == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double x = lane < kThreads / 32 ? sh[k][lane] : 0.0;
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            v[k] = x;
-        }
-    }
-    __syncthreads();
-}
-
-// Block partials without a block-wide barrier at the end: each warp reduces
-// its values with shuffles and parks them in shared memory; the last warp of
-// the block to arrive (a shared arrival counter, zeroed when the kernel
-// starts) adds the warp values in warp order and stores the block partial.
-// Warps that finish early leave at once instead of waiting for the block's
-// slowest gathers.  A one-block finisher kernel launched next sums the block
-// partials in block order: no atomics on floating-point values, no fences on
-// the producers' critical path, a deterministic result.
+// Block partials without a block-wide barrier at the end: every thread parks
+// its values in shared memory; the last warp of the block to arrive (a shared
+// arrival counter, zeroed when the kernel starts) adds them, lane l the
+// values l, l + 32, ... in warp order and then the 32 sums by shuffles, and
+// stores the block partial.  Warps that finish early leave at once instead of
+// waiting for the block's slowest gathers.  A shuffle tree in every warp
+// would issue 40 FP64 warp instructions a block where this issues 12; with
+// eight resident blocks per SM, all ending together, that is 2 us of the FP64
+// pipe at the end of each reducing kernel.  A one-block finisher kernel
+// launched next sums the block partials in block order: no atomics on
+// floating-point values, no fences on the producers' critical path, a
+// deterministic result.
 __device__ __forceinline__ unsigned *arrival_counter() {
     __shared__ unsigned c;
     return &c;
@@ -609,26 +517,23 @@ __device__ __forceinline__ void block_partials_begin() {
 
 template <int NV>
 __device__ __forceinline__ void block_partials(double (&v)[NV], Reduce red) {
-    __shared__ double sh[NV][kThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    double x[NV];
+    __shared__ double sh[NV][kThreads];
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        x[k] = v[k];
-        for (int o = 16; o > 0; o >>= 1) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
-    }
-    if (lane != 0) return;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sh[k][w] = x[k];
+    for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k];
     __threadfence_block();
-    const unsigned nw = blockDim.x >> 5;
-    if (atomicAdd(arrival_counter(), 1u) != nw - 1) return;
+    __syncwarp();
+    unsigned ticket = 0;
+    if (lane == 0) ticket = atomicAdd(arrival_counter(), 1u);
+    if (__shfl_sync(0xffffffffu, ticket, 0) != kThreads / 32 - 1) return;
     __threadfence_block();
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-        double t = 0.0;
-        for (unsigned i = 0; i < nw; ++i) t += ((volatile double *)sh[k])[i];
-        red.partials[k * kMaxReduceBlocks + blockIdx.x] = t;
+        double t = ((volatile double *)sh[k])[lane];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) t += ((volatile double *)sh[k])[lane + 32 * w];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) red.partials[k * kMaxReduceBlocks + blockIdx.x] = t;
     }
 }
 
@@ -751,11 +656,10 @@ ap_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
         const int32_t pos = sl * 32 + lane;
         if (pos >= n) continue;
         const int32_t i = perm ? __ldg(perm + pos) : pos;
-        double s = sell_row_sum<double, double, D16, SHORT, true>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(p + j); });
+        const double s = sell_row_sum<double, double, D16, SHORT, true, RESID>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(p + j); }, RESID ? b[i] : 0.0);
         if (RESID) {
-            const double e = b[i] - s;
-            q[i] = e;
-            part[0] += e * e;
+            q[i] = s;
+            part[0] += s * s;
         } else {
             q[i] = s;
             part[0] += p[i] * s;
@@ -780,10 +684,7 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
         if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
         double s;
         if constexpr (PART) {  // ci: block-local columns
-            const PartRow pr = part_row(pv, i, n, p, nullptr);
-            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t c) {
-                return c < pr.nloc ? __ldg(pr.xl + c) : __ldg(pr.g + (c - pr.nloc));
-            });
+            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, part_row(pv, i, n, p));
         } else {
             s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(p + j); });
         }
@@ -849,17 +750,11 @@ resid_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restric
         int t = (int)(g % T);
         int32_t p0 = 0, p1 = 0;
         if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
-        double s;
-        if constexpr (PART) {
-            const PartRow pr = part_row(pv, i, n, x, nullptr);
-            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t c) {
-                return c < pr.nloc ? __ldg(pr.xl + c) : __ldg(pr.g + (c - pr.nloc));
-            });
-        } else {
-            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); });
-        }
+        const double init = i < n && t == 0 ? b[i] : 0.0;
+        double e;
+        if constexpr (PART) e = csr_row_sum<double, double, T, true>(p0, p1, t, ci, v, part_row(pv, i, n, x), init);
+        else e = csr_row_sum<double, double, T, true>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); }, init);
         if (i < n && t == 0) {
-            double e = b[i] - s;
             t_out[i] = e;
             part[0] += e * e;
         }
@@ -888,18 +783,12 @@ post_rz_csr_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__r
         const int t = (int)(g % T);
         int32_t p0 = 0, p1 = 0;
         if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
-        double s;
-        if constexpr (PART) {
-            const PartRow pr = part_row(pv, i, n, x, nullptr);
-            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t c) {
-                return c < pr.nloc ? __ldg(pr.xl + c) : __ldg(pr.g + (c - pr.nloc));
-            });
-        } else {
-            s = csr_row_sum<double, double, T>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); });
-        }
+        const double bi = i < n && t == 0 ? b[i] : 0.0;
+        double e;
+        if constexpr (PART) e = csr_row_sum<double, double, T, true>(p0, p1, t, ci, v, part_row(pv, i, n, x), bi);
+        else e = csr_row_sum<double, double, T, true>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); }, bi);
         if (i < n && t == 0) {
-            double bi = b[i];
-            double zi = x[i] + dinv[i] * (bi - s);
+            const double zi = x[i] + dinv[i] * e;
             z[i] = zi;
             part[0] += bi * zi;
             if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
@@ -925,9 +814,9 @@ post_rz_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *
         const int32_t pos = sl * 32 + lane;
         if (pos >= n) continue;
         const int32_t i = perm ? __ldg(perm + pos) : pos;
-        double s = sell_row_sum<double, double, D16, false, true>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(x + j); });
-        double bi = b[i];
-        double zi = x[i] + dinv[i] * (bi - s);
+        const double bi = b[i];
+        const double e = sell_row_sum<double, double, D16, false, true, true>(pos, i, soff, sw, ix, sv, [&](int32_t j) { return __ldg(x + j); }, bi);
+        const double zi = x[i] + dinv[i] * e;
         z[i] = zi;
         part[0] += bi * zi;
         if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
@@ -1113,10 +1002,6 @@ int threads_per_row(int variant) {
 }
 
 template <typename VT, typename XT>
-void pre_smooth_residual(const CycMat<VT> &A, const XT *b, const XT *dinv, XT *x, XT *r, cudaStream_t s) {
-    dispatch_op<VT, XT, kPre>(A, b, dinv, nullptr, x, r, s);
-}
-template <typename VT, typename XT>
 void post_smooth(const CycMat<VT> &A, const XT *x, const XT *b, const XT *dinv, XT *xo, cudaStream_t s) {
     dispatch_op<VT, XT, kPost>(A, b, dinv, x, xo, nullptr, s);
 }
@@ -1173,7 +1058,7 @@ static int launch_ap_sell(const CycMat<double> &A, const double *p, const double
 
 void pcg_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc, Reduce red, cudaStream_t s) {
     if (A.part.parts) {  // row-partitioned: exchange, then the one-lane kernel's loop
-        part_exchange(A.part, p, nullptr, s);
+        part_exchange(A.part, p, s);
         const int blocks = reduce_blocks(A.nrows);
         { pdl_launch(ap_kernel<1, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, p, q, sc, red, A.part); ::amg::count_launch(); }
         launch_finish<1, kFinAp>(blocks, red, sc, s);
@@ -1212,7 +1097,7 @@ static void post_smooth_rz_launch(const CycMat<double> &A, const double *x, cons
     const int32_t n = A.nrows;
     constexpr int NV = ZQ ? 2 : 1;
     if (A.part.parts) {
-        part_exchange(A.part, x, nullptr, s);
+        part_exchange(A.part, x, s);
         const int blocks = reduce_blocks(n);
         { pdl_launch(post_rz_csr_kernel<1, ZQ, true>, blocks, kThreads, 0, s, n, A.rp, A.part.cext, A.v, x, b, dinv, z, q, sc, red, A.part); ::amg::count_launch(); }
         launch_finish<NV, kFinRz>(blocks, red, sc, s);
@@ -1285,7 +1170,7 @@ void pcg_rz(int32_t n, const double *r, const double *z, const double *q, PcgSca
 void true_residual(const CycMat<double> &A, const double *b, const double *x, double *t, PcgScalars *sc,
                    Reduce red, cudaStream_t s) {
     if (A.part.parts) {  // row-partitioned: the four-lane kernel's loop, as below
-        part_exchange(A.part, x, nullptr, s);
+        part_exchange(A.part, x, s);
         const int blocks = reduce_blocks((int64_t)A.nrows * 4);
         { pdl_launch(resid_kernel<4, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, b, x, t, sc, red, A.part); ::amg::count_launch(); }
         launch_finish<1, kFinTt>(blocks, red, sc, s);
@@ -1354,7 +1239,6 @@ int32_t max_col_offset(int32_t n, const int32_t *rp, const int32_t *ci, cudaStre
 
 // explicit instantiations
 #define AMG_INST(VT, XT)                                                                                  \
-    template void pre_smooth_residual<VT, XT>(const CycMat<VT> &, const XT *, const XT *, XT *, XT *, cudaStream_t); \
     template void post_smooth<VT, XT>(const CycMat<VT> &, const XT *, const XT *, const XT *, XT *, cudaStream_t); \
     template void spmv<VT, XT>(const CycMat<VT> &, const XT *, XT *, bool, cudaStream_t); \
     template void spmv_scaled<VT, XT>(const CycMat<VT> &, const XT *, const XT *, XT *, XT *, cudaStream_t); \
