@@ -90,7 +90,10 @@ enum { AMG_KRYLOV_CG = 0, AMG_KRYLOV_GMRES = 1 };
 enum { AMG_PREC_FP64 = 0, AMG_PREC_FP32 = 1, AMG_PREC_FP32_BF16 = 2 };
 /* SpMV kernel variants: CSR with T threads per row, or SELL-C slices (C rows
  * per slice, column-major inside it, read by one warp with 32 / C lanes per
- * row: SELL32 one lane per row, SELL16 two, SELL8 four). */
+ * row: SELL32 one lane per row, SELL16 two, SELL8 four).  With AMG_SPMV_AUTO a
+ * finest operator of at most 255 distinct rows (a constant-coefficient stencil)
+ * is stored by them, one byte per row, and read one lane per row in SELL32's
+ * order; it is reported as AMG_SPMV_SELL32. */
 enum {
     AMG_SPMV_AUTO = -1,
     AMG_SPMV_CSR2 = 1, AMG_SPMV_CSR4 = 2, AMG_SPMV_CSR8 = 3, AMG_SPMV_CSR16 = 4,

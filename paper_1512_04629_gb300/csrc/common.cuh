@@ -89,6 +89,7 @@ struct DevBuf {
     ~DevBuf() { release(); }
     void alloc(size_t b);
     void release();
+    void adopt(struct TmpBuf &t);  // takes over t's memory
     template <typename T> T *as() const { return static_cast<T *>(ptr); }
 };
 

@@ -223,6 +223,137 @@ __device__ __forceinline__ XT sell_row_sum(int32_t pos, int32_t row, const int32
     return acc;
 }
 
+// ---------------------------------------------------------------------------
+// Operators stored by row patterns (patterns.cu): the table in shared memory,
+// one lane per row.  What is left to stream is the vectors and one byte per
+// row, so FP64 kernels run at the FP64 pipe and FP32 ones near the bandwidth
+// of the vectors.  A block keeps its table over the rows it takes with the
+// grid's stride, and reads the next row's pattern number while it works on
+// this one.  Against SELL-32 with int16 offsets: 3D 7-point 128^3 in FP64,
+// residual 35.7 -> 29 us (FP64 pipe: 23), post-smoothing with r.z 45.7 -> 38
+// (30), A p 40.4 -> 32 (27); 27-point 192^3, FP32 residual 268 -> 70, FP64
+// A p 391 -> 327 (304).  Six resident blocks per SM: with five the 27-point
+// solve takes 25.2 ms instead of 23.6, with eight (32 registers) 23.8.
+// ---------------------------------------------------------------------------
+#ifndef AMG_PAT_BLOCKS
+#define AMG_PAT_BLOCKS 6
+#endif
+constexpr int kPatBlocks = AMG_PAT_BLOCKS;  // resident blocks per SM the kernels are compiled for
+
+// vectors written by the kernel before: coherent loads that stay behind the
+// dependency wait (a read-only load may be moved above it by the compiler)
+__device__ __forceinline__ double ld_dyn(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_dyn(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
+// The table as the kernels hold it.  FP32 keeps an entry's value and offset
+// side by side, one 8-byte shared load per entry: two loads made the 27-point
+// residual load/store-bound (192^3: 94 -> 72 us).  FP64 keeps two arrays:
+// its kernels are bound by the FP64 pipe, and 16-byte entries cost them more
+// bank conflicts than the second load does (128^3 solve 10.8 vs 10.5 ms).
+template <typename VT> struct PatSmem {
+    const VT *val;         // FP64
+    const int32_t *delta;  // FP64
+    const float2 *ent;     // FP32: value, offset bits
+    const VT *dinv;
+    const int32_t *len;
+    int32_t width;
+    __device__ __forceinline__ void entry(int32_t e, VT &a, int32_t &d) const {
+        if constexpr (sizeof(VT) == 4) {
+            const float2 q = ent[e];
+            a = q.x;
+            d = __float_as_int(q.y);
+        } else {
+            a = val[e];
+            d = delta[e];
+        }
+    }
+};
+
+// copies the table and lets the next kernel launch; returns after this
+// kernel's own predecessor has finished (the table does not depend on it)
+template <typename VT> __device__ __forceinline__ PatSmem<VT> pat_begin(const PatView<VT> &pt) {
+    extern __shared__ __align__(16) unsigned char pat_raw[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int32_t ne = pt.npat * pt.width;
+    VT *val = reinterpret_cast<VT *>(pat_raw);
+    float2 *ent = reinterpret_cast<float2 *>(pat_raw);
+    VT *dinv = sizeof(VT) == 4 ? reinterpret_cast<VT *>(ent + ne) : val + ne;
+    int32_t *len = reinterpret_cast<int32_t *>(dinv + pt.npat), *delta = len + pt.npat;
+    for (int32_t e = threadIdx.x; e < ne; e += kThreads) {
+        const VT a = __ldg(pt.val + e);
+        const int32_t d = __ldg(pt.delta + e);
+        if constexpr (sizeof(VT) == 4) {
+            ent[e] = make_float2(a, __int_as_float(d));
+        } else {
+            val[e] = a;
+            delta[e] = d;
+        }
+    }
+    for (int32_t e = threadIdx.x; e < pt.npat; e += kThreads) {
+        dinv[e] = __ldg(pt.dinv + e);
+        len[e] = __ldg(pt.len + e);
+    }
+    __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return PatSmem<VT>{val, delta, ent, dinv, len, pt.width};
+}
+
+template <int W, bool SUB, typename XT>
+__device__ __forceinline__ XT pat_chunk(XT acc, const PatSmem<XT> &t, int32_t e, const XT *xr) {
+    XT g[W], a[W];
+#pragma unroll
+    for (int k = 0; k < W; ++k) {
+        int32_t d;
+        t.entry(e + k, a[k], d);
+        g[k] = ld_dyn(xr + d);
+    }
+#pragma unroll
+    for (int k = 0; k < W; ++k) acc = mac<SUB>(acc, a[k], g[k]);
+    return acc;
+}
+
+// acc +/- the row's sum, entries in order; the whole warp takes the longest of
+// its rows (the shorter ones add 0 times their own diagonal's x)
+template <bool SUB, typename XT>
+__device__ __forceinline__ XT pat_row_sum(XT acc, const PatSmem<XT> &t, int32_t p, const XT *xr) {
+    const int32_t w = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)t.len[p]);
+    const int32_t e = p * t.width;
+    int32_t k = 0;
+    for (; k + 8 <= w; k += 8) acc = pat_chunk<8, SUB>(acc, t, e + k, xr);
+    switch (w - k) {
+        case 1: return pat_chunk<1, SUB>(acc, t, e + k, xr);
+        case 2: return pat_chunk<2, SUB>(acc, t, e + k, xr);
+        case 3: return pat_chunk<3, SUB>(acc, t, e + k, xr);
+        case 4: return pat_chunk<4, SUB>(acc, t, e + k, xr);
+        case 5: return pat_chunk<5, SUB>(acc, t, e + k, xr);
+        case 6: return pat_chunk<6, SUB>(acc, t, e + k, xr);
+        case 7: return pat_chunk<7, SUB>(acc, t, e + k, xr);
+        default: return acc;
+    }
+}
+
+// f(i, p, live) for every row i of the grid-strided loop, p its pattern; a
+// warp's lanes past the last row repeat it with live = false
+template <typename VT, class F> __device__ __forceinline__ void pat_rows(int32_t n, const PatView<VT> &pt, F f) {
+    const uint32_t stride = gridDim.x * kThreads, last = (uint32_t)n - 1u;  // r + stride < 2^32
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t r = blockIdx.x * kThreads + threadIdx.x;
+    int32_t p = __ldg(pt.pid + min(r, last));
+    for (; r - lane <= last; r += stride) {
+        const int32_t pc = p;
+        p = __ldg(pt.pid + min(r + stride, last));
+        f((int32_t)min(r, last), pc, r <= last);
+    }
+}
+
 enum Op { kPost = 1, kSpmv = 2, kSpmvAdd = 3, kSpmvScale = 4, kResX = 5 };
 
 // the operations that form b - A x: their row accumulators start at b
@@ -291,6 +422,34 @@ sell_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
     } else {
         row_store<XT, OP>(i, s, dinv, x, o1, o2);
     }
+}
+
+template <typename XT, int OP>
+__global__ void __launch_bounds__(kThreads, kPatBlocks)
+pat_op_kernel(int32_t n, PatView<XT> pt, const XT *b, const XT *x, XT *o1, XT *o2) {
+    const PatSmem<XT> t = pat_begin(pt);
+    pat_rows(n, pt, [&](int32_t i, int32_t p, bool live) {
+        const XT xi = OP == kPost ? ld_dyn(x + i) : XT(0);
+        const XT s = pat_row_sum<kIsResid<OP>>(kIsResid<OP> ? ld_dyn(b + i) : XT(0), t, p, x + i);
+        if (!live) return;
+        if (OP == kPost) o1[i] = xi + t.dinv[p] * s;
+        else if (OP == kSpmv) o1[i] = s;
+        else o2[i] = s;
+    });
+}
+
+// rows in rounds of one resident wave, the blocks spread evenly over them
+static int pat_grid(int32_t n) {
+    const int64_t need = div_up((int64_t)n, (int64_t)kThreads), res = ::amg::resident_blocks(2048) * (int64_t)kPatBlocks;
+    return (int)div_up(need, div_up(need, res));
+}
+
+template <typename XT, int OP>
+static void launch_pat_op(const CycMat<XT> &A, const XT *b, const XT *x, XT *o1, XT *o2, cudaStream_t s) {
+    const size_t smem = pat_smem_bytes<XT>(A.pat.npat, A.pat.width);
+    pdl_launch(pat_op_kernel<XT, OP>, pat_grid(A.nrows), kThreads, smem, s, A.nrows, A.pat, b, x, o1, o2);
+    ::amg::count_launch();
+    AMG_CHECK_LAUNCH();
 }
 
 // ---------------------------------------------------------------------------
@@ -441,6 +600,12 @@ void dispatch_op(const CycMat<VT> &A, const XT *b, const XT *dinv, const XT *x, 
     if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
         if (A.part.parts) {
             part_op<OP>(A, b, dinv, x, o1, o2, s);
+            return;
+        }
+    }
+    if constexpr (std::is_same<VT, XT>::value && (kIsResid<OP> || OP == kSpmv)) {
+        if (A.pat.pid) {
+            launch_pat_op<XT, OP>(A, b, x, o1, o2, s);
             return;
         }
     }
@@ -668,6 +833,23 @@ ap_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
     block_partials<1>(part, red);
 }
 
+// the same with the operator stored by row patterns
+template <bool RESID>
+__global__ void __launch_bounds__(kThreads, kPatBlocks)
+ap_pat_kernel(int32_t n, PatView<double> pt, const double *p, const double *b, double *q, PcgScalars *sc, Reduce red) {
+    block_partials_begin();
+    const PatSmem<double> t = pat_begin(pt);
+    double part[1] = {0.0};
+    pat_rows(n, pt, [&](int32_t i, int32_t pat, bool live) {
+        const double pi = RESID ? 0.0 : ld_dyn(p + i);
+        const double s = pat_row_sum<RESID>(RESID ? ld_dyn(b + i) : 0.0, t, pat, p + i);
+        if (!live) return;
+        q[i] = s;
+        part[0] += RESID ? s * s : pi * s;
+    });
+    block_partials<1>(part, red);
+}
+
 // q = A p (vector-CSR, T lanes per row) and p . q
 template <int T, bool PART = false>
 __global__ void __launch_bounds__(kThreads)
@@ -821,6 +1003,27 @@ post_rz_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *
         part[0] += bi * zi;
         if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
     }
+    block_partials<ZQ ? 2 : 1>(part, red);
+}
+
+template <bool ZQ>
+__global__ void __launch_bounds__(kThreads, kPatBlocks)
+post_rz_pat_kernel(int32_t n, PatView<double> pt, const double *x, const double *b, double *z, const double *q,
+                   PcgScalars *sc, Reduce red) {
+    block_partials_begin();
+    const PatSmem<double> t = pat_begin(pt);
+    double part[ZQ ? 2 : 1];
+#pragma unroll
+    for (int k = 0; k < (ZQ ? 2 : 1); ++k) part[k] = 0.0;
+    pat_rows(n, pt, [&](int32_t i, int32_t p, bool live) {
+        const double bi = ld_dyn(b + i), xi = ld_dyn(x + i);
+        const double e = pat_row_sum<true>(bi, t, p, x + i);
+        if (!live) return;
+        const double zi = xi + t.dinv[p] * e;
+        z[i] = zi;
+        part[0] += bi * zi;
+        if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
+    });
     block_partials<ZQ ? 2 : 1>(part, red);
 }
 
@@ -1065,6 +1268,13 @@ void pcg_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc,
         AMG_CHECK_LAUNCH();
         return;
     }
+    if (A.pat.pid) {
+        const int blocks = pat_grid(A.nrows);
+        { pdl_launch(ap_pat_kernel<false>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, p, (const double *)nullptr, q, sc, red); ::amg::count_launch(); }
+        launch_finish<1, kFinAp>(blocks, red, sc, s);
+        AMG_CHECK_LAUNCH();
+        return;
+    }
     if (A.variant == AMG_SPMV_SELL32 && A.sv && A.sell_c == 32) {
         const int blocks = launch_ap_sell<false>(A, p, nullptr, q, sc, red, s);
         launch_finish<1, kFinAp>(blocks, red, sc, s);
@@ -1100,6 +1310,13 @@ static void post_smooth_rz_launch(const CycMat<double> &A, const double *x, cons
         part_exchange(A.part, x, s);
         const int blocks = reduce_blocks(n);
         { pdl_launch(post_rz_csr_kernel<1, ZQ, true>, blocks, kThreads, 0, s, n, A.rp, A.part.cext, A.v, x, b, dinv, z, q, sc, red, A.part); ::amg::count_launch(); }
+        launch_finish<NV, kFinRz>(blocks, red, sc, s);
+        AMG_CHECK_LAUNCH();
+        return;
+    }
+    if (A.pat.pid) {
+        const int blocks = pat_grid(n);
+        { pdl_launch(post_rz_pat_kernel<ZQ>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, n, A.pat, x, b, z, q, sc, red); ::amg::count_launch(); }
         launch_finish<NV, kFinRz>(blocks, red, sc, s);
         AMG_CHECK_LAUNCH();
         return;
@@ -1173,6 +1390,13 @@ void true_residual(const CycMat<double> &A, const double *b, const double *x, do
         part_exchange(A.part, x, s);
         const int blocks = reduce_blocks((int64_t)A.nrows * 4);
         { pdl_launch(resid_kernel<4, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, b, x, t, sc, red, A.part); ::amg::count_launch(); }
+        launch_finish<1, kFinTt>(blocks, red, sc, s);
+        AMG_CHECK_LAUNCH();
+        return;
+    }
+    if (A.pat.pid) {
+        const int blocks = pat_grid(A.nrows);
+        { pdl_launch(ap_pat_kernel<true>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, x, b, t, sc, red); ::amg::count_launch(); }
         launch_finish<1, kFinTt>(blocks, red, sc, s);
         AMG_CHECK_LAUNCH();
         return;

@@ -24,6 +24,23 @@ struct PartView {
     int64_t nghost = 0;
 };
 
+// An operator of few distinct rows (patterns.cu): the pattern of each row and
+// the patterns' entries as column offsets from the row and values, `width`
+// slots each (past a pattern's length: value 0 at offset 0).
+template <typename VT> struct PatView {
+    const uint8_t *pid = nullptr;  // null: not stored by patterns
+    const int32_t *len = nullptr, *delta = nullptr;
+    const VT *val = nullptr, *dinv = nullptr;  // dinv: the row's inverse ell1 diagonal
+    int32_t npat = 0, width = 0;
+};
+constexpr int kPatMax = 255, kPatWidth = 32;
+// shared memory of a pattern kernel's table; kPatSmem: the largest accepted,
+// so that the blocks of a full SM and the L1 cache share it (27-point: 9 KB)
+template <typename VT> inline size_t pat_smem_bytes(int32_t npat, int32_t width) {
+    return (size_t)npat * ((size_t)(width + 1) * (sizeof(VT) + sizeof(int32_t)));
+}
+constexpr size_t kPatSmem = 12 * 1024;
+
 // A matrix as the cycle kernels read it: CSR in value type VT, plus an
 // optional SELL-C copy (slices of C rows, column-major inside a slice).
 template <typename VT> struct CycMat {
@@ -43,6 +60,7 @@ template <typename VT> struct CycMat {
                           // with the evict-first policy (read once per pass, they would only
                           // push the vectors and the smaller levels out of L1 and L2)
     PartView part;        // set when the hierarchy runs row-partitioned (FP64 only)
+    PatView<VT> pat;      // set when the operator has few distinct rows (level 0; FP64 and FP32)
 };
 constexpr int64_t kStreamBytes = 48ll << 20;
 
@@ -142,6 +160,20 @@ template <typename VT>
 void sell_fill(int32_t n, const int32_t *rp, const int32_t *ci, const VT *v, const int32_t *perm,
                const int32_t *soff, const int32_t *sw, int32_t *sci, VT *sv, cudaStream_t s, int16_t *sd = nullptr,
                int C = 32);
+// the device table of the patterns, in one allocation of pat_table_bytes()
+struct PatTable {
+    double *val64, *dinv64;
+    float *val32, *dinv32;
+    int32_t *delta, *len;
+};
+size_t pat_table_bytes();
+PatTable pat_table(void *base);
+// M by its distinct rows: pid (n bytes) and the table; false when there are
+// more than kPatMax, a row is empty or longer than kPatWidth, or the table
+// would pass kPatSmem (pid and table then hold nothing of use).  dinv: the
+// inverse ell1 diagonal, a function of the row's values.
+bool build_patterns(const DevCSR &M, const double *dinv, uint8_t *pid, void *table, int32_t *npat, int32_t *width,
+                    cudaStream_t s);
 // max over stored entries of |column - row| (square operators), for the int16 SELL offsets;
 // *max_row (if given) receives the longest row
 int32_t max_col_offset(int32_t n, const int32_t *rp, const int32_t *ci, cudaStream_t s, int32_t *max_row = nullptr);

@@ -406,6 +406,8 @@ template <typename VT> static void build_sell(Level &V, cudaStream_t s, int C = 
 static void free_sell(Level &V) {
     V.soff.release(); V.sw.release(); V.sci.release(); V.sd.release(); V.sv.release(); V.sperm.release();
     V.sv64.release();
+    V.pid.release(); V.ptab.release();
+    V.npat = V.pwidth = 0;
     V.sell_entries = 0;
 }
 
@@ -583,6 +585,21 @@ static bool prepare_level_at(Hierarchy &h, Level &V, int l, bool has_p, cudaStre
         if (it != g_tune_cache.end()) {
             V.variant = it->second;
             tune = false;
+        }
+    }
+    // The finest operator of few distinct rows is stored by them (patterns.cu)
+    // and read one lane per row in row order, as SELL-32: nothing to time.
+    // Coarse operators are never that regular, and a forced variant is used
+    // as given.  Below the tuning threshold a cycle is launch latency alone.
+    if (l == 0 && forced == AMG_SPMV_AUTO && M.nnz >= 20000 && has_p) {
+        // temporaries until they are known to serve: a persistent buffer's
+        // release would wait for the whole device, the coarsening included
+        TmpBuf pid(n + kPad, s), tab(cyc::pat_table_bytes(), s);
+        if (cyc::build_patterns(M, V.dinv.as<double>(), pid.as<uint8_t>(), tab.ptr, &V.npat, &V.pwidth, s)) {
+            V.pid.adopt(pid);
+            V.ptab.adopt(tab);
+            V.variant = AMG_SPMV_SELL32;
+            return false;
         }
     }
     if (tune && !allow_tune) return true;
@@ -1200,6 +1217,7 @@ CycMat<double> a0_mat(Hierarchy &h) {
         return m;
     }
     CycMat<double> m = make_mat<double>(V.A, V.A.v());
+    m.pat = pat_view<double>(V);
     if (V.variant == AMG_SPMV_SELL32 && V.sv64.ptr) {
         m.variant = AMG_SPMV_SELL32;
         m.nslices = (V.A.nrows + 31) / 32;

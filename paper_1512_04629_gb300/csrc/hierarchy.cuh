@@ -73,6 +73,8 @@ struct Level {
     DevBuf sd;                 // its columns as int16 offsets from the row (instead of sci) when they fit
     DevBuf sperm;              // SELL position -> row when rows are length-sorted
     DevBuf sv64;               // level 0 in FP32 modes: FP64 values in the same SELL layout (outer PCG)
+    DevBuf pid, ptab;          // level 0 with few distinct rows: pattern of each row, the patterns (npat > 0)
+    int32_t npat = 0, pwidth = 0;
     int64_t sell_entries = 0;
     int sell_c = 32;
     int32_t max_row = 0;       // longest row of the relaxed operator (kernel choice)
@@ -194,6 +196,23 @@ template <typename VT> inline CycMat<VT> make_mat(const DevCSR &M, const VT *val
     return m;
 }
 
+// the pattern storage of a level's relaxed operator (pid null without one)
+template <typename VT> inline PatView<VT> pat_view(const Level &V) {
+    PatView<VT> p;
+    if constexpr (sizeof(VT) >= 4) {
+        if (V.npat == 0) return p;
+        const cyc::PatTable t = cyc::pat_table(V.ptab.ptr);
+        p.pid = V.pid.as<uint8_t>();
+        p.len = t.len;
+        p.delta = t.delta;
+        if constexpr (sizeof(VT) == 8) { p.val = t.val64; p.dinv = t.dinv64; }
+        else { p.val = t.val32; p.dinv = t.dinv32; }
+        p.npat = V.npat;
+        p.width = V.pwidth;
+    }
+    return p;
+}
+
 template <typename VT> inline CycMat<VT> op_mat(const Level &V) {
     const DevCSR &M = V.op();
     const VT *vals;
@@ -213,6 +232,7 @@ template <typename VT> inline CycMat<VT> op_mat(const Level &V) {
     }
     m.max_row = V.max_row;
     m.variant = V.variant;
+    m.pat = pat_view<VT>(V);
     if constexpr (sizeof(VT) == 8)
         if (V.part_h) m.part = V.part_h->view();
     return m;

@@ -136,6 +136,14 @@ void DevBuf::alloc(size_t b) {
     bytes = b;
     g_device_bytes += (int64_t)b;
 }
+void DevBuf::adopt(TmpBuf &t) {
+    release();
+    ptr = t.ptr;
+    bytes = t.bytes;
+    t.ptr = nullptr;
+    t.bytes = 0;
+    g_device_bytes += (int64_t)bytes;
+}
 void DevBuf::release() {
     if (ptr) {
         cudaStream_t ps = nullptr;
