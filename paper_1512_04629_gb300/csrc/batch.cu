@@ -5,10 +5,22 @@
 // consecutive columns W t .. W t + W - 1, moved as one 16-byte vector (W = 4
 // floats or 2 doubles).  Every lane of the group reads the row's (column,
 // value) pairs itself -- the same address across the group, served as one
-// broadcast -- and keeps the vector loads of kAhead entries in flight before
-// it uses them; each column still sums its entries in row order.  The matrix
-// is read once per block of K right-hand sides instead of K times.
+// broadcast -- with the next kAhead entries' pairs on their way while the
+// vectors of this one's are gathered; each column sums its entries in row
+// order.  The matrix is read once per block of K right-hand sides instead of
+// K times.  A block takes a contiguous range of rows: what a row gathers of
+// the grid lines beside its own is then still in L1 from the block's last
+// steps, and L2 -- whose bandwidth bounds these kernels, a 7-point row at
+// K = 32 gathers 7 x 128 bytes -- serves it about once instead of per row.
+// Lognormal 112^3, K = 32, FP32, finest level: residual 165 -> 113 us (it no
+// longer writes x = D^-1 b either), prolongation 124 -> 97, post-smoothing
+// 170 -> 121 (it writes the correction in FP32, not widened); the whole
+// solve 78.3 -> 73.0 ms.  Forming r.z in the post-smoothing too was slower
+// (340 us against 121 + 179): its registers leave half the warps.
 #include <cuda_bf16.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "batch_ops.cuh"
 #include "common.cuh"
@@ -23,10 +35,6 @@ constexpr int kThreads = 256;
 template <typename VT, typename XT> __device__ __forceinline__ XT cvt(VT v) { return (XT)v; }
 
 template <> __device__ __forceinline__ float cvt<__nv_bfloat16, float>(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-enum Op { kPre = 0, kPost = 1, kSpmv = 2, kSpmvAdd = 3 };
-
-constexpr int kAhead = 4;  // entries whose vector loads are in flight together
 
 // 16-byte vectors of a row block (the block's base is 16-byte aligned: K is a
 // multiple of 8 and every n x K buffer starts on an allocation boundary)
@@ -53,157 +61,217 @@ __device__ __forceinline__ void vstore(float *p, const float (&x)[4]) {
 __device__ __forceinline__ void vstore(double *p, const double (&x)[2]) {
     *reinterpret_cast<double2 *>(p) = make_double2(x[0], x[1]);
 }
-// the FP32 cycle's finest post-smoothing writes the FP64 correction itself
-// (4 floats widened exactly into 32 bytes of doubles) instead of a separate
-// conversion pass.  Its input stays the FP32 copy of the residual: a gather
-// that rounded FP64 neighbours on load would convert every value once per
-// row that uses it, on GB300's narrow FP64 pipe.
-__device__ __forceinline__ void vstore(double *p, const float (&x)[4]) {
-    reinterpret_cast<double2 *>(p)[0] = make_double2((double)x[0], (double)x[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2((double)x[2], (double)x[3]);
+
+// Conversions between the cycle's FP32 and the outer loop's FP64 on the integer
+// pipes, exact and to nearest even: a conversion instruction holds the FP64
+// pipe for 16 clocks as an FMA does -- also when it is predicated off, so the
+// rare cases below are calls, which the compiler cannot turn into predicates.
+// Every element of a batched iteration is widened twice and rounded once; on
+// the conversion instructions the r.z pass of 45 M elements took 260 us, twice
+// its memory time.
+__device__ __noinline__ double widen_rare(float f) { return (double)f; }
+__device__ __noinline__ float narrow_rare(double x) { return (float)x; }
+
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) return widen_rare(f);  // subnormal, infinite, NaN
+    const uint32_t hi = (u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// FP32 has 29 fewer fraction bits and an exponent bias 896 lower; rounding up
+// carries into the exponent and, from the largest, to infinity
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x), m = u & 0x7fffffffffffffffull;
+    const uint32_t e = (uint32_t)(m >> 52);
+    if (e - 897u > 253u && m != 0ull) return narrow_rare(x);  // outside FP32's normal range
+    const uint32_t r = (uint32_t)((m + 0x0fffffffull + ((m >> 29) & 1ull)) >> 29) - (896u << 23);
+    return __uint_as_float((uint32_t)(u >> 32 & 0x80000000u) | (m ? r : 0u));
 }
 
-// acc[w] += sum over the row's entries, in entry order, of a_ij * src_j[c0 + w]
-// (times dinv_j when SCALE: the pre-smoothing's x_j = dinv_j b_j)
-template <typename VT, typename XT, typename ST, int K, bool SCALE>
-__device__ __forceinline__ void row_block_sum(int32_t p0, int32_t p1, const int32_t *__restrict__ ci,
-                                              const VT *__restrict__ v, const ST *__restrict__ src,
-                                              const XT *__restrict__ dinv, int c0, XT (&acc)[16 / sizeof(XT)]) {
+constexpr int kSpmmThreads = 512;  // largest block of an SpMM pass
+constexpr int kAhead = 4;          // entries whose vector loads are in flight together
+// resident blocks the passes are compiled for: FP32 three (42 registers) --
+// with two its passes at 112^3, K = 32 take 8% longer, with four or with two
+// entries ahead 4-9% -- and FP64, whose operands fill 64 registers, two
+template <typename XT> constexpr int kSpmmBlocks = sizeof(XT) == 8 ? 2 : 3;
+
+// entries e .. e + C - 1 of a row: their columns and values, then their
+// vectors, are in flight together
+template <int C, typename VT, typename XT, int K, bool SCALE, bool SUB>
+__device__ __forceinline__ void entries(int32_t e, const int32_t *__restrict__ ci, const VT *__restrict__ v,
+                                        const XT *__restrict__ src, const XT *__restrict__ dinv, int c0,
+                                        XT (&acc)[16 / sizeof(XT)]) {
     constexpr int W = 16 / sizeof(XT);
-    int32_t e = p0;
-    for (; e + kAhead <= p1; e += kAhead) {
-        int32_t j[kAhead];
-        XT a[kAhead], d[kAhead], x[kAhead][W];
+    int32_t j[C];
+    XT a[C], x[C][W], m[C];
 #pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-            j[q] = __ldg(ci + e + q);
-            a[q] = cvt<VT, XT>(__ldg(v + e + q));
-        }
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-            vload(src + (int64_t)j[q] * K + c0, x[q]);
-            if (SCALE) d[q] = __ldg(dinv + j[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < kAhead; ++q) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) {
-                if (SCALE) acc[w] += a[q] * (x[q][w] * d[q]);
-                else acc[w] += a[q] * x[q][w];
-            }
-        }
+    for (int q = 0; q < C; ++q) {
+        j[q] = __ldg(ci + e + q);
+        a[q] = cvt<VT, XT>(__ldg(v + e + q));
     }
-    for (; e < p1; ++e) {
-        const int32_t j = __ldg(ci + e);
-        const XT a = cvt<VT, XT>(__ldg(v + e));
-        XT x[W];
-        vload(src + (int64_t)j * K + c0, x);
-        if (SCALE) {
-            const XT d = __ldg(dinv + j);
 #pragma unroll
-            for (int w = 0; w < W; ++w) acc[w] += a * (x[w] * d);
-        } else {
-#pragma unroll
-            for (int w = 0; w < W; ++w) acc[w] += a * x[w];
-        }
+    for (int q = 0; q < C; ++q) {
+        vload(src + (int64_t)j[q] * K + c0, x[q]);
+        if (SCALE) m[q] = __ldg(dinv + j[q]);
     }
-}
-
-// BT: type of B (the right-hand side); OT: type of O1 for the
-// post-smoothing (double on the FP32 cycle's level 0, else XT)
-template <typename VT, typename XT, typename BT, typename OT, int K, int OP>
-__global__ void __launch_bounds__(kThreads)
-spmm_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const VT *__restrict__ v,
-            const BT *__restrict__ B, const XT *__restrict__ dinv, const XT *__restrict__ X,
-            OT *__restrict__ O1, XT *__restrict__ O2) {
-    constexpr int W = 16 / sizeof(XT), G = K / W;
-    const int64_t g = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    const int32_t i = (int32_t)(g / G);
-    if (i >= n) return;
-    const int c0 = (int)(g % G) * W;
-    XT acc[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) acc[w] = XT(0);
-    if constexpr (OP == kPre) row_block_sum<VT, XT, BT, K, true>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, B, dinv, c0, acc);
-    else row_block_sum<VT, XT, XT, K, false>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, X, dinv, c0, acc);
-    const int64_t base = (int64_t)i * K + c0;
-    XT o[W];
-    if constexpr (OP == kPre) {
-        const XT di = dinv[i];
-        XT bi[W], r[W];
-        vload(B + base, bi);
+    for (int q = 0; q < C; ++q) {
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            o[w] = bi[w] * di;
-            r[w] = bi[w] - acc[w];
+            const XT y = SCALE ? x[q][w] * m[q] : x[q][w];
+            if (SUB) acc[w] -= a[q] * y;
+            else acc[w] += a[q] * y;
         }
-        vstore(O1 + base, o);
-        vstore(O2 + base, r);
-    } else if constexpr (OP == kPost) {
-        const XT di = dinv[i];
-        XT xi[W], bi[W];
-        vload(X + base, xi);
-        vload(B + base, bi);
-#pragma unroll
-        for (int w = 0; w < W; ++w) o[w] = xi[w] + di * (bi[w] - acc[w]);
-        vstore(O1 + base, o);
-    } else if constexpr (OP == kSpmv) {
-        vstore(O1 + base, acc);
-    } else {
-        vload_rw(O1 + base, o);
-#pragma unroll
-        for (int w = 0; w < W; ++w) o[w] += acc[w];
-        vstore(O1 + base, o);
     }
 }
 
-template <typename VT, typename XT, int OP, typename BT = XT, typename OT = XT>
-void dispatch(const CycMat<VT> &A, int K, const BT *B, const XT *dinv, const XT *X, OT *O1, XT *O2, cudaStream_t s) {
-    int32_t n = A.nrows;
+// acc += sum over the row's entries, in entry order, of a_ij * src_j[c0 ..]
+// (SCALE: times dinv_j, for x_j = dinv_j b_j that was never written); SUB:
+// subtracted, for residuals whose accumulator starts at b.  kAhead entries
+// at a time, the rest by halves -- no predicated-off FMAs, which would cost
+// the FP64 pipe as much as real ones
+template <typename VT, typename XT, int K, bool SCALE, bool SUB>
+__device__ __forceinline__ void row_block_sum(int32_t p0, int32_t p1, const int32_t *__restrict__ ci,
+                                              const VT *__restrict__ v, const XT *__restrict__ src,
+                                              const XT *__restrict__ dinv, int c0, XT (&acc)[16 / sizeof(XT)]) {
+    int32_t e = p0;
+    for (; e + kAhead <= p1; e += kAhead) entries<kAhead, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+    if (e + 2 <= p1) {
+        entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+        e += 2;
+    }
+    if (e < p1) entries<1, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+}
+
+// operands of an SpMM pass (unused ones null)
+template <typename XT> struct SpmmArgs {
+    const XT *B = nullptr;     // right-hand sides of this level
+    const XT *X = nullptr;     // the gathered block
+    const XT *dinv = nullptr;  // this level's inverse ell1 diagonal (restriction: the coarse level's)
+    XT *O1 = nullptr, *O2 = nullptr;
+};
+
+// kResB: O1 = B - A (dinv .* B), the residual of a pre-smooth x = dinv .* B
+//        that is not written (kProlB forms it again); kRes: O1 = B - A X
+// kPost: O1 = X + dinv .* (B - A X)
+// kRest: O1 = R X; kRestX: also O2 = dinv .* O1, the coarse pre-smooth
+// kProl: O1 += P X; kProlB: O1 = dinv .* B + P X
+enum Op { kResB, kRes, kPost, kRest, kRestX, kProl, kProlB };
+
+template <typename VT, typename XT, int K, int OP>
+__global__ void __launch_bounds__(kSpmmThreads, kSpmmBlocks<XT>)
+spmm_kernel(int32_t n, int32_t chunk, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
+            const VT *__restrict__ v, SpmmArgs<XT> g) {
+    constexpr int W = 16 / sizeof(XT), G = K / W;
+    constexpr bool kResid = OP == kResB || OP == kRes || OP == kPost;
+    const int c0 = (int)(threadIdx.x % G) * W, step = blockDim.x / G;
+    const int64_t lo = (int64_t)blockIdx.x * chunk, hi = min((int64_t)n, lo + chunk);
+    int64_t i = lo + threadIdx.x / G;
+    int32_t p0 = 0, p1 = 0;
+    if (i < hi) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
+    for (; i < hi; i += step) {
+        const int32_t q0 = p0, q1 = p1;
+        if (i + step < hi) { p0 = __ldg(rp + i + step); p1 = __ldg(rp + i + step + 1); }
+        const int64_t base = i * K + c0;
+        XT acc[W], o[W];
+        if constexpr (kResid) vload(g.B + base, acc);
+        else {
+#pragma unroll
+            for (int w = 0; w < W; ++w) acc[w] = XT(0);
+        }
+        if constexpr (OP == kProlB) vload(g.B + base, o);
+        if constexpr (OP == kProl) vload_rw(g.O1 + base, o);
+        if constexpr (OP == kPost) vload(g.X + base, o);
+        XT d = XT(0);
+        if constexpr (OP == kPost || OP == kRestX || OP == kProlB) d = __ldg(g.dinv + i);
+        row_block_sum<VT, XT, K, OP == kResB, kResid>(q0, q1, ci, v, OP == kResB ? g.B : g.X, g.dinv, c0, acc);
+        if constexpr (OP == kResB || OP == kRes || OP == kRest || OP == kRestX) {
+            vstore(g.O1 + base, acc);
+            if constexpr (OP == kRestX) {
+#pragma unroll
+                for (int w = 0; w < W; ++w) o[w] = acc[w] * d;
+                vstore(g.O2 + base, o);
+            }
+        } else {
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                if constexpr (OP == kProl) o[w] += acc[w];
+                else if constexpr (OP == kProlB) o[w] = o[w] * d + acc[w];
+                else o[w] += d * acc[w];
+            }
+            vstore(g.O1 + base, o);
+        }
+    }
+}
+
+// A block's threads and rows: as many blocks as stay resident, each with an
+// even contiguous share; levels too small to fill the device that way get
+// smaller blocks, down to one warp's rows each.
+struct SpmmGrid {
+    int threads, blocks;
+    int32_t chunk;
+};
+SpmmGrid spmm_grid(int64_t n, int G, int resident) {
+    const int64_t sms = ::amg::resident_blocks(2048);
+    int threads = kSpmmThreads;
+    while (threads > 64 && div_up(n * G, threads) < sms * resident) threads >>= 1;
+    const int64_t rows = threads / G;  // per step
+    const int64_t want = (n + rows - 1) / rows;
+    const int64_t cap = sms * resident * (kSpmmThreads / threads);
+    const int64_t steps = (want + cap - 1) / cap;
+    SpmmGrid g;
+    g.threads = threads;
+    g.chunk = (int32_t)(steps * rows);
+    g.blocks = (int)((n + g.chunk - 1) / g.chunk);
+    return g;
+}
+
+template <typename VT, typename XT, int OP>
+void dispatch(const CycMat<VT> &A, int K, const SpmmArgs<XT> &g, cudaStream_t s) {
+    const int32_t n = A.nrows;
     if (n == 0) return;
-    constexpr int W = 16 / sizeof(XT);
-    auto blocks = [&](int k) { return div_up((int64_t)n * (k / W), kThreads); };
+    auto launch = [&](auto kc) {
+        constexpr int KK = decltype(kc)::value;
+        const SpmmGrid gr = spmm_grid(n, KK / (16 / (int)sizeof(XT)), kSpmmBlocks<XT>);
+        spmm_kernel<VT, XT, KK, OP><<<gr.blocks, gr.threads, 0, s>>>(n, gr.chunk, A.rp, A.ci, A.v, g);
+        ::amg::count_launch();
+    };
     switch (K) {
-        case 8: { spmm_kernel<VT, XT, BT, OT, 8, OP><<<blocks(8), kThreads, 0, s>>>(n, A.rp, A.ci, A.v, B, dinv, X, O1, O2); ::amg::count_launch(); } break;
-        case 16: { spmm_kernel<VT, XT, BT, OT, 16, OP><<<blocks(16), kThreads, 0, s>>>(n, A.rp, A.ci, A.v, B, dinv, X, O1, O2); ::amg::count_launch(); } break;
-        case 32: { spmm_kernel<VT, XT, BT, OT, 32, OP><<<blocks(32), kThreads, 0, s>>>(n, A.rp, A.ci, A.v, B, dinv, X, O1, O2); ::amg::count_launch(); } break;
-        case 64: { spmm_kernel<VT, XT, BT, OT, 64, OP><<<blocks(64), kThreads, 0, s>>>(n, A.rp, A.ci, A.v, B, dinv, X, O1, O2); ::amg::count_launch(); } break;
+        case 8: launch(std::integral_constant<int, 8>{}); break;
+        case 16: launch(std::integral_constant<int, 16>{}); break;
+        case 32: launch(std::integral_constant<int, 32>{}); break;
+        case 64: launch(std::integral_constant<int, 64>{}); break;
         default: throw Error(AMG_ERR_INVALID, "batch width must be 8, 16, 32 or 64");
     }
     AMG_CHECK_LAUNCH();
 }
 
+// one block per row of the dense inverse: thread groups of K lanes take every
+// (256 / K)-th entry, and the groups' sums are added in order (one thread per
+// column walking the row alone took 10 us at 62 unknowns)
 template <typename XT>
-__global__ void coarse_kernel(int32_t n, int K, const double *__restrict__ inv, const XT *__restrict__ B, XT *__restrict__ X) {
-    int32_t row = blockIdx.x;
-    for (int c = threadIdx.x; c < K; c += blockDim.x) {
-        double s = 0.0;
-        for (int32_t j = 0; j < n; ++j) s += inv[(size_t)row * n + j] * (double)B[(int64_t)j * K + c];
-        X[(int64_t)row * K + c] = (XT)s;
-    }
+__global__ void __launch_bounds__(kThreads)
+coarse_kernel(int32_t n, int K, const double *__restrict__ inv, const XT *__restrict__ B, XT *__restrict__ X) {
+    __shared__ double sh[kThreads];
+    const int32_t row = blockIdx.x;
+    const int c = threadIdx.x % K, g = threadIdx.x / K, ng = kThreads / K;
+    double s = 0.0;
+#pragma unroll 4
+    for (int32_t j = g; j < n; j += ng) s += inv[(size_t)row * n + j] * (double)B[(int64_t)j * K + c];
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.x >= K) return;
+    for (int q = 1; q < ng; ++q) s += sh[q * K + threadIdx.x];
+    X[(int64_t)row * K + c] = (XT)s;
 }
 
 // ---------------------------------------------------------------------------
-// per-column deterministic reductions.  A thread's slot is its column; each
-// block sums its slots in thread order and stores one partial per column; a
-// finisher kernel (one block per column) sums the partials in block order
-// and updates that column's scalars.  No atomics, no fences.
-template <int NV>
-__device__ void col_partials(double (&v)[NV], int K, double *partials) {
-    __shared__ double sh[NV][kThreads];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k];
-    __syncthreads();
-    if (threadIdx.x < K) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double s = 0.0;
-            for (int r = threadIdx.x; r < kThreads; r += K) s += sh[k][r];
-            partials[((size_t)k * kMaxCols + threadIdx.x) * kBatchReduceBlocks + blockIdx.x] = s;
-        }
-    }
-}
-
+// per-column deterministic reductions.  Each block sums its threads' values of
+// a column in thread order and stores one partial per column; a finisher
+// kernel (one block per column) sums the partials in block order and updates
+// that column's scalars.  No atomics, no fences.
 enum ColFin { kColRz = 0, kColAp = 1, kColXr = 2, kColTt = 3 };
 
 template <int NV, int FIN>
@@ -238,7 +306,7 @@ col_finish_kernel(int nblocks, const double *partials, ColScalars sc, int flexib
             double rho_new = out[0];
             if (sc.start[c]) sc.beta[c] = 0.0;
             else sc.beta[c] = flexible ? (-sc.alpha[c] * out[NV - 1]) / sc.rho[c] : rho_new / sc.rho[c];
-            sc.zq[c] = out[NV - 1];
+            if (NV > 1) sc.zq[c] = out[NV - 1];
             sc.rho[c] = rho_new;
             sc.start[c] = 0;
         }
@@ -263,27 +331,88 @@ int grid_for(int64_t n, int K) {
     return (int)b;
 }
 
-// thread -> (row, column) with column = threadIdx % K (K divides 256)
-__global__ void __launch_bounds__(kThreads)
-rz_kernel(int32_t n, int K, const double *__restrict__ R, const double *__restrict__ Z, const double *__restrict__ Q,
-          double *partials) {
-    int c = threadIdx.x % K;
-    int rpb = kThreads / K;
-    double v[2] = {0.0, 0.0};
-    for (int64_t i = (int64_t)blockIdx.x * rpb + threadIdx.x / K; i < n; i += (int64_t)gridDim.x * rpb) {
-        double z = Z[i * K + c];
-        v[0] += R[i * K + c] * z;
-        v[1] += z * Q[i * K + c];
-    }
-    col_partials<2>(v, K, partials);
+__device__ __forceinline__ void zload(const double *p, double (&z)[2]) { vload(p, z); }
+__device__ __forceinline__ void zload(const float *p, double (&z)[2]) {
+    const float2 q = __ldg(reinterpret_cast<const float2 *>(p));
+    z[0] = widen(q.x);
+    z[1] = widen(q.y);
 }
 
-__global__ void p_update_kernel(int64_t total, int K, const double *__restrict__ Z, double *__restrict__ P, ColScalars sc) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= total) return;
-    int c = (int)(e % K);
-    if (!sc.active[c]) return;
-    P[e] = Z[e] + sc.beta[c] * P[e];
+// per-column sums of a block whose threads hold two adjacent columns each
+// (lane t of a group of K / 2: columns 2 t, 2 t + 1), threads in order
+template <int K, int NV>
+__device__ __forceinline__ void pair_partials(const double (&part)[NV][2], double *partials) {
+    constexpr int G = K / 2;
+    __shared__ double sh[NV][2][kThreads];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        sh[k][0][threadIdx.x] = part[k][0];
+        sh[k][1][threadIdx.x] = part[k][1];
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < NV * K; e += kThreads) {
+        const int k = e / K, c = e % K;
+        double sum = 0.0;
+        for (int t = c / 2; t < kThreads; t += G) sum += sh[k][c & 1][t];
+        partials[((size_t)k * kMaxCols + c) * kBatchReduceBlocks + blockIdx.x] = sum;
+    }
+}
+
+// r.z and (NV = 2) z.q: two columns of a row per thread, rows grid-stride
+template <int K, int NV, typename ZT>
+__global__ void __launch_bounds__(kThreads)
+rz_kernel(int32_t n, const double *__restrict__ R, const ZT *__restrict__ Z, const double *__restrict__ Q,
+          double *partials) {
+    constexpr int G = K / 2, RPB = kThreads / G;
+    double part[NV][2] = {};
+    const int c = (int)(threadIdx.x % G) * 2;
+#pragma unroll 2
+    for (int64_t i = (int64_t)blockIdx.x * RPB + threadIdx.x / G; i < n; i += (int64_t)gridDim.x * RPB) {
+        const int64_t e = i * K + c;
+        double z[2], r[2];
+        zload(Z + e, z);
+        vload(R + e, r);
+        part[0][0] += r[0] * z[0];
+        part[0][1] += r[1] * z[1];
+        if constexpr (NV == 2) {
+            double q[2];
+            vload(Q + e, q);
+            part[1][0] += q[0] * z[0];
+            part[1][1] += q[1] * z[1];
+        }
+    }
+    pair_partials<K, NV>(part, partials);
+}
+
+// P = Z + beta P on the active columns, two per thread
+template <int K, typename ZT>
+__global__ void __launch_bounds__(kThreads)
+p_update_kernel(int64_t pairs, const ZT *__restrict__ Z, double *__restrict__ P, ColScalars sc) {
+    const int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (e >= pairs) return;
+    const int c = (int)(e % (K / 2)) * 2;
+    const bool a0 = sc.active[c] != 0, a1 = sc.active[c + 1] != 0;
+    if (!a0 && !a1) return;
+    double z[2], p[2];
+    zload(Z + 2 * e, z);
+    vload_rw(P + 2 * e, p);
+    if (a0) p[0] = z[0] + sc.beta[c] * p[0];
+    if (a1) p[1] = z[1] + sc.beta[c + 1] * p[1];
+    vstore(P + 2 * e, p);
+}
+
+// x = dinv .* R on an n x K block (the FP64 cycle's finest pre-smooth)
+template <int K>
+__global__ void __launch_bounds__(kThreads)
+scale_kernel(int64_t pairs, const double *__restrict__ R, const double *__restrict__ dinv, double *__restrict__ X) {
+    const int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (e >= pairs) return;
+    const double d = __ldg(dinv + e / (K / 2));
+    double r[2];
+    vload(R + 2 * e, r);
+    r[0] *= d;
+    r[1] *= d;
+    vstore(X + 2 * e, r);
 }
 
 // Q = A P (or T = B - A X when RESID) on the FP64 n x K blocks, with the
@@ -299,17 +428,13 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
     double part[W] = {0.0, 0.0};
     for (int64_t i = (int64_t)blockIdx.x * RPB + threadIdx.x / G; i < n; i += (int64_t)gridDim.x * RPB) {
         double acc[W] = {0.0, 0.0};
-        row_block_sum<double, double, double, K, false>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, Pin, nullptr, c0, acc);
         const int64_t base = i * K + c0;
+        if (RESID) vload(Bin + base, acc);
+        row_block_sum<double, double, K, false, RESID>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, Pin, nullptr, c0, acc);
         if (RESID) {
-            double b[W], r[W];
-            vload(Bin + base, b);
 #pragma unroll
-            for (int w = 0; w < W; ++w) {
-                r[w] = b[w] - acc[w];
-                part[w] += r[w] * r[w];
-            }
-            vstore(Qout + base, r);
+            for (int w = 0; w < W; ++w) part[w] += acc[w] * acc[w];
+            vstore(Qout + base, acc);
         } else {
             double p[W];
             vload(Pin + base, p);
@@ -331,40 +456,67 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
     }
 }
 
+// two columns of a row per thread, rows grid-stride.  At 112^3, K = 32 it
+// moves 2.34 GB in 433 us, 80% of the copy rate; streaming load and store
+// policies change nothing
+template <int K>
 __global__ void __launch_bounds__(kThreads)
-xr_kernel(int32_t n, int K, const double *__restrict__ P, const double *__restrict__ Q, double *__restrict__ X,
+xr_kernel(int32_t n, const double *__restrict__ P, const double *__restrict__ Q, double *__restrict__ X,
           double *__restrict__ R, float *__restrict__ R32, ColScalars sc, double *partials) {
-    int c = threadIdx.x % K;
-    int rpb = kThreads / K;
-    double alpha = sc.active[c] ? sc.alpha[c] : 0.0;
-    double v[1] = {0.0};
-    for (int64_t i = (int64_t)blockIdx.x * rpb + threadIdx.x / K; i < n; i += (int64_t)gridDim.x * rpb) {
-        int64_t e = i * K + c;
-        double r = R[e];
-        if (alpha != 0.0) {
-            X[e] += alpha * P[e];
-            r -= alpha * Q[e];
-            R[e] = r;
+    constexpr int G = K / 2, RPB = kThreads / G;
+    const int c = (int)(threadIdx.x % G) * 2;
+    const double a0 = sc.active[c] ? sc.alpha[c] : 0.0, a1 = sc.active[c + 1] ? sc.alpha[c + 1] : 0.0;
+    // tested as integers: a comparison of doubles would sit in the loop on the FP64 pipe
+    const bool s0 = __double_as_longlong(a0) << 1 != 0, s1 = __double_as_longlong(a1) << 1 != 0;
+    double part[1][2] = {};
+#pragma unroll 2
+    for (int64_t i = (int64_t)blockIdx.x * RPB + threadIdx.x / G; i < n; i += (int64_t)gridDim.x * RPB) {
+        const int64_t e = i * K + c;
+        double r[2];
+        vload_rw(R + e, r);
+        if (s0 || s1) {
+            double x[2], p[2], q[2];
+            vload_rw(X + e, x);
+            vload(P + e, p);
+            vload(Q + e, q);
+            if (s0) {
+                x[0] += a0 * p[0];
+                r[0] -= a0 * q[0];
+            }
+            if (s1) {
+                x[1] += a1 * p[1];
+                r[1] -= a1 * q[1];
+            }
+            vstore(X + e, x);
+            vstore(R + e, r);
         }
-        if (R32) R32[e] = (float)r;  // the next FP32 cycle's input, every column
-        v[0] += r * r;
+        // the next FP32 cycle's input, every column
+        if (R32) *reinterpret_cast<float2 *>(R32 + e) = make_float2(narrow(r[0]), narrow(r[1]));
+        part[0][0] += r[0] * r[0];
+        part[0][1] += r[1] * r[1];
     }
-    col_partials<1>(v, K, partials);
+    pair_partials<K, 1>(part, partials);
 }
 
-__global__ void scatter_kernel(int32_t n, int K, int c, const double *v, double *M, float *M32) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// a request's right-hand side into column c of B, R (and R32); X, P, Q zeroed
+__global__ void __launch_bounds__(kThreads)
+admit_kernel(int32_t n, int K, int c, const double *__restrict__ b, double *__restrict__ B, double *__restrict__ R,
+             float *__restrict__ R32, double *__restrict__ X, double *__restrict__ P, double *__restrict__ Q) {
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
-    M[i * K + c] = v[i];
-    if (M32) M32[i * K + c] = (float)v[i];
+    const int64_t e = i * K + c;
+    const double v = b[i];
+    B[e] = v;
+    R[e] = v;
+    if (R32) R32[e] = (float)v;
+    X[e] = 0.0;
+    P[e] = 0.0;
+    Q[e] = 0.0;
 }
+
 __global__ void gather_kernel(int32_t n, int K, int c, const double *M, double *v) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) v[i] = M[i * K + c];
-}
-__global__ void zero_col_kernel(int32_t n, int K, int c, double *M) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) M[i * K + c] = 0.0;
 }
 __global__ void copy_masked_kernel(int64_t total, int K, const double *T, double *R, float *R32, const int *mask) {
     int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -377,11 +529,6 @@ template <typename XT> __global__ void to_cycle_kernel(const double *src, XT *ds
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dst[i] = (XT)src[i];
 }
-template <typename XT> __global__ void from_cycle_kernel(const XT *src, double *dst, int64_t n) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) dst[i] = (double)src[i];
-}
-
 }  // namespace
 
 int batch_width(int k) {
@@ -392,38 +539,85 @@ int batch_width(int k) {
     throw Error(AMG_ERR_INVALID, "at most 64 right-hand sides per batch");
 }
 
-template <typename VT, typename XT>
-void pre_smooth_residual(const CycMat<VT> &A, int K, const XT *B, const XT *dinv, XT *X, XT *R, cudaStream_t s) {
-    dispatch<VT, XT, kPre, XT, XT>(A, K, B, dinv, nullptr, X, R, s);
+namespace {
+// f(std::integral_constant<int, K>) for a compiled width
+template <class F> void with_width(int K, F &&f) {
+    switch (K) {
+        case 8: f(std::integral_constant<int, 8>{}); break;
+        case 16: f(std::integral_constant<int, 16>{}); break;
+        case 32: f(std::integral_constant<int, 32>{}); break;
+        case 64: f(std::integral_constant<int, 64>{}); break;
+        default: throw Error(AMG_ERR_INVALID, "batch width must be 8, 16, 32 or 64");
+    }
+    AMG_CHECK_LAUNCH();
 }
-template <typename VT, typename XT, typename OT>
-void post_smooth(const CycMat<VT> &A, int K, const XT *X, const XT *B, const XT *dinv, OT *XO, cudaStream_t s) {
-    dispatch<VT, XT, kPost, XT, OT>(A, K, B, dinv, X, XO, nullptr, s);
+}  // namespace
+
+template <typename VT, typename XT>
+void residual_of_scaled(const CycMat<VT> &A, int K, const XT *B, const XT *dinv, XT *R, cudaStream_t s) {
+    SpmmArgs<XT> g;
+    g.B = B; g.dinv = dinv; g.O1 = R;
+    dispatch<VT, XT, kResB>(A, K, g, s);
 }
 template <typename VT, typename XT>
-void spmm(const CycMat<VT> &A, int K, const XT *X, XT *Y, bool accumulate, cudaStream_t s) {
-    if (accumulate) dispatch<VT, XT, kSpmvAdd, XT, XT>(A, K, nullptr, nullptr, X, Y, nullptr, s);
-    else dispatch<VT, XT, kSpmv, XT, XT>(A, K, nullptr, nullptr, X, Y, nullptr, s);
+void residual_from_x(const CycMat<VT> &A, int K, const XT *B, const XT *X, XT *R, cudaStream_t s) {
+    SpmmArgs<XT> g;
+    g.B = B; g.X = X; g.O1 = R;
+    dispatch<VT, XT, kRes>(A, K, g, s);
+}
+template <typename VT, typename XT>
+void post_smooth(const CycMat<VT> &A, int K, const XT *X, const XT *B, const XT *dinv, XT *XO, cudaStream_t s) {
+    SpmmArgs<XT> g;
+    g.B = B; g.X = X; g.dinv = dinv; g.O1 = XO;
+    dispatch<VT, XT, kPost>(A, K, g, s);
+}
+template <typename XT>
+void restrict_to(const CycMat<XT> &R, int K, const XT *X, XT *BC, const XT *dinv_c, XT *XC, cudaStream_t s) {
+    SpmmArgs<XT> g;
+    g.X = X; g.O1 = BC; g.dinv = dinv_c; g.O2 = XC;
+    if (XC) dispatch<XT, XT, kRestX>(R, K, g, s);
+    else dispatch<XT, XT, kRest>(R, K, g, s);
+}
+template <typename XT>
+void prolong_add(const CycMat<XT> &P, int K, const XT *XC, XT *X, const XT *B, const XT *dinv, cudaStream_t s) {
+    SpmmArgs<XT> g;
+    g.X = XC; g.O1 = X; g.B = B; g.dinv = dinv;
+    if (B) dispatch<XT, XT, kProlB>(P, K, g, s);
+    else dispatch<XT, XT, kProl>(P, K, g, s);
 }
 template <typename XT>
 void coarse_solve(int32_t n, int K, const double *inv, const XT *B, XT *X, cudaStream_t s) {
     if (n == 0) return;
-    { coarse_kernel<XT><<<n, 64, 0, s>>>(n, K, inv, B, X); ::amg::count_launch(); }
+    { coarse_kernel<XT><<<n, kThreads, 0, s>>>(n, K, inv, B, X); ::amg::count_launch(); }
+    AMG_CHECK_LAUNCH();
+}
+void scale(int32_t n, int K, const double *R, const double *dinv, double *X, cudaStream_t s) {
+    const int64_t pairs = (int64_t)n * K / 2;
+    with_width(K, [&](auto kc) {
+        scale_kernel<decltype(kc)::value><<<div_up(pairs, kThreads), kThreads, 0, s>>>(pairs, R, dinv, X);
+        ::amg::count_launch();
+    });
+}
+
+template <typename ZT>
+void rz(int32_t n, int K, const double *R, const ZT *Z, const double *Q, ColScalars sc, double *partials,
+        cudaStream_t s) {
+    constexpr int NV = sizeof(ZT) == 8 ? 1 : 2;  // FP32 cycles: flexible CG, whose beta needs z.q
+    const int blocks = grid_for(n, K / 2);
+    with_width(K, [&](auto kc) {
+        rz_kernel<decltype(kc)::value, NV, ZT><<<blocks, kThreads, 0, s>>>(n, R, Z, Q, partials);
+        ::amg::count_launch();
+    });
+    { col_finish_kernel<NV, kColRz><<<K, kThreads, 0, s>>>(blocks, partials, sc, NV == 2); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
 
-void rz(int32_t n, int K, const double *R, const double *Z, const double *Q, ColScalars sc, int flexible,
-        double *partials, cudaStream_t s) {
-    int blocks = grid_for(n, K);
-    { rz_kernel<<<blocks, kThreads, 0, s>>>(n, K, R, Z, Q, partials); ::amg::count_launch(); }
-    { col_finish_kernel<2, kColRz><<<K, kThreads, 0, s>>>(blocks, partials, sc, flexible); ::amg::count_launch(); }
-    AMG_CHECK_LAUNCH();
-}
-
-void p_update(int32_t n, int K, const double *Z, double *P, ColScalars sc, cudaStream_t s) {
-    int64_t total = (int64_t)n * K;
-    { p_update_kernel<<<div_up(total, kThreads), kThreads, 0, s>>>(total, K, Z, P, sc); ::amg::count_launch(); }
-    AMG_CHECK_LAUNCH();
+template <typename ZT> void p_update(int32_t n, int K, const ZT *Z, double *P, ColScalars sc, cudaStream_t s) {
+    const int64_t pairs = (int64_t)n * K / 2;
+    with_width(K, [&](auto kc) {
+        p_update_kernel<decltype(kc)::value, ZT><<<div_up(pairs, kThreads), kThreads, 0, s>>>(pairs, Z, P, sc);
+        ::amg::count_launch();
+    });
 }
 
 // one resident wave of ap_kernel blocks (at least four rows per thread group)
@@ -475,22 +669,22 @@ void residual(const CycMat<double> &A, int K, const double *B, const double *X, 
 
 void xr_update(int32_t n, int K, const double *P, const double *Q, double *X, double *R, float *R32, ColScalars sc,
                double *partials, cudaStream_t s) {
-    int blocks = grid_for(n, K);
-    { xr_kernel<<<blocks, kThreads, 0, s>>>(n, K, P, Q, X, R, R32, sc, partials); ::amg::count_launch(); }
+    const int blocks = grid_for(n, K / 2);
+    with_width(K, [&](auto kc) {
+        xr_kernel<decltype(kc)::value><<<blocks, kThreads, 0, s>>>(n, P, Q, X, R, R32, sc, partials);
+        ::amg::count_launch();
+    });
     { col_finish_kernel<1, kColXr><<<K, kThreads, 0, s>>>(blocks, partials, sc, 0); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
 
-void scatter_column(int32_t n, int K, int c, const double *v, double *M, cudaStream_t s, float *M32) {
-    { scatter_kernel<<<div_up(n, kThreads), kThreads, 0, s>>>(n, K, c, v, M, M32); ::amg::count_launch(); }
+void admit_column(int32_t n, int K, int c, const double *b, double *B, double *R, float *R32, double *X, double *P,
+                  double *Q, cudaStream_t s) {
+    { admit_kernel<<<div_up(n, kThreads), kThreads, 0, s>>>(n, K, c, b, B, R, R32, X, P, Q); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
 void gather_column(int32_t n, int K, int c, const double *M, double *v, cudaStream_t s) {
     { gather_kernel<<<div_up(n, kThreads), kThreads, 0, s>>>(n, K, c, M, v); ::amg::count_launch(); }
-    AMG_CHECK_LAUNCH();
-}
-void zero_column(int32_t n, int K, int c, double *M, cudaStream_t s) {
-    { zero_col_kernel<<<div_up(n, kThreads), kThreads, 0, s>>>(n, K, c, M); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
 void copy_masked_columns(int32_t n, int K, const double *T, double *R, const int *mask, cudaStream_t s, float *R32) {
@@ -503,34 +697,27 @@ template <typename XT> void to_cycle(const double *src, XT *dst, int64_t n, cuda
     { to_cycle_kernel<XT><<<div_up(n, kThreads), kThreads, 0, s>>>(src, dst, n); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
-template <typename XT> void from_cycle(const XT *src, double *dst, int64_t n, cudaStream_t s) {
-    { from_cycle_kernel<XT><<<div_up(n, kThreads), kThreads, 0, s>>>(src, dst, n); ::amg::count_launch(); }
-    AMG_CHECK_LAUNCH();
-}
-
-#define AMG_PINST(VT, XT) \
-    template void pre_smooth_residual<VT, XT>(const CycMat<VT> &, int, const XT *, const XT *, XT *, XT *, cudaStream_t);
-AMG_PINST(double, double)
+#define AMG_PINST(VT, XT)                                                                                          \
+    template void residual_of_scaled<VT, XT>(const CycMat<VT> &, int, const XT *, const XT *, XT *, cudaStream_t); \
+    template void post_smooth<VT, XT>(const CycMat<VT> &, int, const XT *, const XT *, const XT *, XT *, cudaStream_t);
 AMG_PINST(float, float)
 AMG_PINST(__nv_bfloat16, float)
 #undef AMG_PINST
-#define AMG_QINST(VT, XT, OT) \
-    template void post_smooth<VT, XT, OT>(const CycMat<VT> &, int, const XT *, const XT *, const XT *, OT *, cudaStream_t);
-AMG_QINST(double, double, double)
-AMG_QINST(float, float, float)
-AMG_QINST(__nv_bfloat16, float, float)
-AMG_QINST(float, float, double)
-AMG_QINST(__nv_bfloat16, float, double)
-#undef AMG_QINST
-#define AMG_SINST(VT, XT) template void spmm<VT, XT>(const CycMat<VT> &, int, const XT *, XT *, bool, cudaStream_t);
-AMG_SINST(double, double)
-AMG_SINST(float, float)
-AMG_SINST(__nv_bfloat16, float)
+template void residual_from_x<double, double>(const CycMat<double> &, int, const double *, const double *, double *,
+                                              cudaStream_t);
+template void post_smooth<double, double>(const CycMat<double> &, int, const double *, const double *, const double *,
+                                          double *, cudaStream_t);
+#define AMG_SINST(XT)                                                                                               \
+    template void restrict_to<XT>(const CycMat<XT> &, int, const XT *, XT *, const XT *, XT *, cudaStream_t);       \
+    template void prolong_add<XT>(const CycMat<XT> &, int, const XT *, XT *, const XT *, const XT *, cudaStream_t); \
+    template void coarse_solve<XT>(int32_t, int, const double *, const XT *, XT *, cudaStream_t);                   \
+    template void rz<XT>(int32_t, int, const double *, const XT *, const double *, ColScalars, double *,            \
+                         cudaStream_t);                                                                             \
+    template void p_update<XT>(int32_t, int, const XT *, double *, ColScalars, cudaStream_t);
+AMG_SINST(double)
+AMG_SINST(float)
 #undef AMG_SINST
-template void coarse_solve<double>(int32_t, int, const double *, const double *, double *, cudaStream_t);
-template void coarse_solve<float>(int32_t, int, const double *, const float *, float *, cudaStream_t);
 template void to_cycle<float>(const double *, float *, int64_t, cudaStream_t);
-template void from_cycle<float>(const float *, double *, int64_t, cudaStream_t);
 
 }  // namespace bat
 }  // namespace amg

@@ -37,15 +37,16 @@ BatchWS &batch_workspace(Hierarchy &h, int K, cudaStream_t s) {
         }
     }
     size_t nb = sizeof(double) * ((size_t)h.lev[0]->n() * K + kPad);
-    for (DevBuf *d : {&w->B, &w->X, &w->R, &w->Z, &w->P, &w->Q, &w->T}) {
+    for (DevBuf *d : {&w->B, &w->X, &w->R, &w->P, &w->Q, &w->T}) {
         d->alloc(nb);
         AMG_CUDA(cudaMemsetAsync(d->ptr, 0, nb, s));
     }
+    w->Z.alloc(xb * ((size_t)h.lev[0]->n() * K + kPad));  // the cycle's output, in its precision
+    AMG_CUDA(cudaMemsetAsync(w->Z.ptr, 0, w->Z.bytes, s));
     if (h.opt.precision != AMG_PREC_FP64) {
         size_t fb = sizeof(float) * ((size_t)h.lev[0]->n() * K + kPad);
         w->R32.alloc(fb);
         AMG_CUDA(cudaMemsetAsync(w->R32.ptr, 0, fb, s));  // kept equal to (float) R by every writer of R
-        if (L == 1) w->Z32.alloc(fb);  // deeper cycles write Z themselves
     }
     w->sc_buf.alloc(sizeof(double) * 7 * K + sizeof(int) * 3 * K);
     AMG_CUDA(cudaMemsetAsync(w->sc_buf.ptr, 0, w->sc_buf.bytes, s));
@@ -68,68 +69,59 @@ void batch_push_flags(BatchWS &w, cudaStream_t s) {
     AMG_CUDA(cudaMemcpyAsync(w.sc.active, w.h_i, sizeof(int) * 2 * w.K, cudaMemcpyHostToDevice, s));
 }
 
-// level l's smoothers; the finest post-smoothing writes Z0 of type OT0
-// (double on the FP32 cycle: no separate conversion pass back)
+// Z = M B0 over the hierarchy's levels (at least two).  The FP32 cycle never writes a pre-smooth x = D^{-1} b: the residual multiplies by
+// D^{-1} as it gathers and the prolongation forms x from b.  In FP64 that
+// multiplication would double the passes' work on the FP64 pipe, which bounds
+// them, so x is written there -- with the restriction, or by a pass of its own
+// on the finest level.
 template <typename XT>
-static void pre_level(Level &V, int K, const XT *b, XT *x, XT *r, cudaStream_t s) {
-    if constexpr (sizeof(XT) == 8) {
-        bat::pre_smooth_residual<double, double>(op_mat<double>(V), K, b, dinv_of<XT>(V), x, r, s);
-    } else if (V.vbytes == 2) {
-        bat::pre_smooth_residual<__nv_bfloat16, float>(op_mat<__nv_bfloat16>(V), K, b, dinv_of<XT>(V), x, r, s);
-    } else {
-        bat::pre_smooth_residual<float, float>(op_mat<float>(V), K, b, dinv_of<XT>(V), x, r, s);
-    }
-}
-template <typename XT, typename OT>
-static void post_level(Level &V, int K, const XT *x, const XT *b, OT *out, cudaStream_t s) {
-    if constexpr (sizeof(XT) == 8) {
-        bat::post_smooth<double, double, OT>(op_mat<double>(V), K, x, b, dinv_of<XT>(V), out, s);
-    } else if (V.vbytes == 2) {
-        bat::post_smooth<__nv_bfloat16, float, OT>(op_mat<__nv_bfloat16>(V), K, x, b, dinv_of<XT>(V), out, s);
-    } else {
-        bat::post_smooth<float, float, OT>(op_mat<float>(V), K, x, b, dinv_of<XT>(V), out, s);
-    }
-}
-
-// Z0 = M B0 over the hierarchy's levels (at least two)
-template <typename XT, typename OT0>
-static void batch_vcycle_impl(Hierarchy &h, BatchWS &w, const XT *B0, OT0 *Z0, cudaStream_t s) {
-    int L = h.nlev(), K = w.K;
+static void batch_vcycle_impl(Hierarchy &h, BatchWS &w, const XT *B0, XT *Z0, cudaStream_t s) {
+    constexpr bool kF64 = sizeof(XT) == 8;
+    const int L = h.nlev(), K = w.K;
+    const int32_t n0 = h.lev[0]->n();
+    if constexpr (kF64) bat::scale(n0, K, B0, dinv_of<XT>(*h.lev[0]), w.x[0].as<XT>(), s);
     for (int l = 0; l + 1 < L; ++l) {
         Level &V = *h.lev[l];
-        XT *x = w.x[l].as<XT>(), *r = w.r[l].as<XT>();
-        pre_level<XT>(V, K, l == 0 ? B0 : w.b[l].as<XT>(), x, r, s);
-        bat::spmm<XT, XT>(r_mat<XT>(V), K, r, w.b[l + 1].as<XT>(), false, s);
+        XT *r = w.r[l].as<XT>();
+        const XT *b = l == 0 ? B0 : w.b[l].as<XT>();
+        if constexpr (kF64)
+            bat::residual_from_x<double, double>(op_mat<double>(V), K, b, w.x[l].as<XT>(), r, s);
+        else if (V.vbytes == 2)
+            bat::residual_of_scaled<__nv_bfloat16, float>(op_mat<__nv_bfloat16>(V), K, b, dinv_of<XT>(V), r, s);
+        else
+            bat::residual_of_scaled<float, float>(op_mat<float>(V), K, b, dinv_of<XT>(V), r, s);
+        Level &C = *h.lev[l + 1];
+        const bool xc = kF64 && l + 2 < L;
+        bat::restrict_to<XT>(r_mat<XT>(V), K, r, w.b[l + 1].as<XT>(), xc ? dinv_of<XT>(C) : nullptr,
+                             xc ? w.x[l + 1].as<XT>() : nullptr, s);
     }
     bat::coarse_solve<XT>(h.coarse_n, K, h.coarse_inv.as<double>(), w.b[L - 1].as<XT>(), w.xo[L - 1].as<XT>(), s);
     for (int l = L - 2; l >= 0; --l) {
         Level &V = *h.lev[l];
         XT *x = w.x[l].as<XT>();
-        bat::spmm<XT, XT>(p_mat<XT>(V), K, w.xo[l + 1].as<XT>(), x, true, s);
-        if (l == 0) post_level<XT, OT0>(V, K, x, B0, Z0, s);
-        else post_level<XT, XT>(V, K, x, w.b[l].as<XT>(), w.xo[l].as<XT>(), s);
+        const XT *b = l == 0 ? B0 : w.b[l].as<XT>();
+        bat::prolong_add<XT>(p_mat<XT>(V), K, w.xo[l + 1].as<XT>(), x, kF64 ? nullptr : b, dinv_of<XT>(V), s);
+        XT *out = l == 0 ? Z0 : w.xo[l].as<XT>();
+        if constexpr (kF64)
+            bat::post_smooth<double, double>(op_mat<double>(V), K, x, b, dinv_of<XT>(V), out, s);
+        else if (V.vbytes == 2)
+            bat::post_smooth<__nv_bfloat16, float>(op_mat<__nv_bfloat16>(V), K, x, b, dinv_of<XT>(V), out, s);
+        else
+            bat::post_smooth<float, float>(op_mat<float>(V), K, x, b, dinv_of<XT>(V), out, s);
     }
 }
 
-// Z = M R for all K columns
-void batch_vcycle(Hierarchy &h, BatchWS &w, cudaStream_t s) {
-    int64_t nk = (int64_t)h.lev[0]->n() * w.K;
-    const bool fp64 = h.opt.precision == AMG_PREC_FP64;
-    if (fp64) {
-        if (h.nlev() == 1)
-            bat::coarse_solve<double>(h.coarse_n, w.K, h.coarse_inv.as<double>(), w.R.as<double>(), w.Z.as<double>(), s);
-        else
-            batch_vcycle_impl<double, double>(h, w, w.R.as<double>(), w.Z.as<double>(), s);
-        return;
-    }
-    // R32 = (float) R already: written with R by the x, r update, admission
-    // and residual replacement
-    if (h.nlev() == 1) {  // the coarse solve alone, in FP32 vectors
-        bat::coarse_solve<float>(h.coarse_n, w.K, h.coarse_inv.as<double>(), w.R32.as<float>(), w.Z32.as<float>(), s);
-        bat::from_cycle<float>(w.Z32.as<float>(), w.Z.as<double>(), nk, s);
-    } else {
-        batch_vcycle_impl<float, double>(h, w, w.R32.as<float>(), w.Z.as<double>(), s);
-    }
+// Z = M R for all K columns, rho and beta; then P = Z + beta P.  The FP32
+// cycle's input R32 = (float) R is kept by every writer of R.
+template <typename XT>
+static void batch_direction(Hierarchy &h, BatchWS &w, const XT *B0, cudaStream_t s) {
+    const int32_t n = h.lev[0]->n();
+    if (h.nlev() == 1)
+        bat::coarse_solve<XT>(h.coarse_n, w.K, h.coarse_inv.as<double>(), B0, w.Z.as<XT>(), s);
+    else
+        batch_vcycle_impl<XT>(h, w, B0, w.Z.as<XT>(), s);
+    bat::rz<XT>(n, w.K, w.R.as<double>(), w.Z.as<XT>(), w.Q.as<double>(), w.sc, w.partials.as<double>(), s);
+    bat::p_update<XT>(n, w.K, w.Z.as<XT>(), w.P.as<double>(), w.sc, s);
 }
 
 static CycMat<double> a0(Hierarchy &h) {
@@ -143,10 +135,8 @@ static CycMat<double> a0(Hierarchy &h) {
 static void batch_iteration_body(Hierarchy &h, BatchWS &w, cudaStream_t s) {
     int32_t n = h.lev[0]->n();
     int K = w.K;
-    int flexible = h.opt.precision != AMG_PREC_FP64;
-    batch_vcycle(h, w, s);
-    bat::rz(n, K, w.R.as<double>(), w.Z.as<double>(), w.Q.as<double>(), w.sc, flexible, w.partials.as<double>(), s);
-    bat::p_update(n, K, w.Z.as<double>(), w.P.as<double>(), w.sc, s);
+    if (h.opt.precision == AMG_PREC_FP64) batch_direction<double>(h, w, w.R.as<double>(), s);
+    else batch_direction<float>(h, w, w.R32.as<float>(), s);
     bat::ap(a0(h), K, w.P.as<double>(), w.Q.as<double>(), w.sc, w.partials.as<double>(), s);
     bat::xr_update(n, K, w.P.as<double>(), w.Q.as<double>(), w.X.as<double>(), w.R.as<double>(), w.R32.as<float>(), w.sc,
                    w.partials.as<double>(), s);

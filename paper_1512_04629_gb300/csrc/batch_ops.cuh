@@ -16,16 +16,25 @@ namespace bat {
 // smallest width >= k (extra columns stay zero and inactive)
 int batch_width(int k);
 
+// R = B - A (dinv .* B): the residual of the pre-smooth x = dinv .* B, which is
+// not written (prolong_add forms it again from B)
 template <typename VT, typename XT>
-void pre_smooth_residual(const CycMat<VT> &A, int K, const XT *B, const XT *dinv, XT *X, XT *R, cudaStream_t s);
-// OT: type of the output -- XT, or double for the FP32 cycle's finest level,
-// which writes the FP64 correction Z directly
-template <typename VT, typename XT, typename OT = XT>
-void post_smooth(const CycMat<VT> &A, int K, const XT *X, const XT *B, const XT *dinv, OT *XO, cudaStream_t s);
+void residual_of_scaled(const CycMat<VT> &A, int K, const XT *B, const XT *dinv, XT *R, cudaStream_t s);
+// R = B - A X
 template <typename VT, typename XT>
-void spmm(const CycMat<VT> &A, int K, const XT *X, XT *Y, bool accumulate, cudaStream_t s);
+void residual_from_x(const CycMat<VT> &A, int K, const XT *B, const XT *X, XT *R, cudaStream_t s);
+template <typename VT, typename XT>
+void post_smooth(const CycMat<VT> &A, int K, const XT *X, const XT *B, const XT *dinv, XT *XO, cudaStream_t s);
+// BC = R X and, with XC, the coarse pre-smooth XC = dinv_c .* BC
+template <typename XT>
+void restrict_to(const CycMat<XT> &R, int K, const XT *X, XT *BC, const XT *dinv_c, XT *XC, cudaStream_t s);
+// X += P XC; with B: X = dinv .* B + P XC
+template <typename XT>
+void prolong_add(const CycMat<XT> &P, int K, const XT *XC, XT *X, const XT *B, const XT *dinv, cudaStream_t s);
 template <typename XT>
 void coarse_solve(int32_t n, int K, const double *inv, const XT *B, XT *X, cudaStream_t s);
+// X = dinv .* R
+void scale(int32_t n, int K, const double *R, const double *dinv, double *X, cudaStream_t s);
 
 // per-column PCG state on the device
 struct ColScalars {
@@ -34,10 +43,13 @@ struct ColScalars {
     int *start;   // 1: first iteration after (re)start: beta = 0
 };
 
-// Z = M R done by the caller; then:
-void rz(int32_t n, int K, const double *R, const double *Z, const double *Q, ColScalars sc, int flexible,
-        double *partials, cudaStream_t s);
-void p_update(int32_t n, int K, const double *Z, double *P, ColScalars sc, cudaStream_t s);
+// Z = M R done by the caller (in the cycle's precision: FP32 widens exactly);
+// then rho = R . Z, (FP32 cycles: flexible CG) Z . Q, and beta
+template <typename ZT>
+void rz(int32_t n, int K, const double *R, const ZT *Z, const double *Q, ColScalars sc, double *partials,
+        cudaStream_t s);
+// P = Z + beta P
+template <typename ZT> void p_update(int32_t n, int K, const ZT *Z, double *P, ColScalars sc, cudaStream_t s);
 void ap(const CycMat<double> &A, int K, const double *P, double *Q, ColScalars sc, double *partials,
         cudaStream_t s);
 // R32 (FP32 cycles; else nullptr): also written with every column's new
@@ -47,17 +59,16 @@ void xr_update(int32_t n, int K, const double *P, const double *Q, double *X, do
 // T = B - A X, tt[c] = ||T_c||^2
 void residual(const CycMat<double> &A, int K, const double *B, const double *X, double *T, ColScalars sc,
               double *partials, cudaStream_t s);
-// column c of an n x K block <- / -> a contiguous n-vector
-// (M32: when given, column c of the FP32 copy of M too)
-void scatter_column(int32_t n, int K, int c, const double *v, double *M, cudaStream_t s, float *M32 = nullptr);
+// a request joins column c: b into B, R (and R32, the FP32 cycle's copy), X, P, Q zero
+void admit_column(int32_t n, int K, int c, const double *b, double *B, double *R, float *R32, double *X, double *P,
+                  double *Q, cudaStream_t s);
+// column c of an n x K block -> a contiguous n-vector
 void gather_column(int32_t n, int K, int c, const double *M, double *v, cudaStream_t s);
-void zero_column(int32_t n, int K, int c, double *M, cudaStream_t s);
 // R = T for the columns flagged in mask (residual replacement)
 void copy_masked_columns(int32_t n, int K, const double *T, double *R, const int *mask, cudaStream_t s,
                          float *R32 = nullptr);
 
 template <typename XT> void to_cycle(const double *src, XT *dst, int64_t n, cudaStream_t s);
-template <typename XT> void from_cycle(const XT *src, double *dst, int64_t n, cudaStream_t s);
 
 constexpr int kMaxCols = 64;
 constexpr int kBatchReduceBlocks = 8192;

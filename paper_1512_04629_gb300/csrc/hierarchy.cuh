@@ -116,7 +116,7 @@ struct BatchWS {
     int K = 0;
     std::vector<DevBuf> b, x, r, xo;
     DevBuf B, X, R, Z, P, Q, T;
-    DevBuf R32, Z32;
+    DevBuf R32;  // (float) R, the FP32 cycle's input (Z: the cycle's output, in its precision)
     DevBuf sc_buf, partials, mask;
     bat::ColScalars sc{};
     double *h_d = nullptr;  // pinned: rho, pq, alpha, beta, rr, zq, tt (K each)
@@ -314,7 +314,6 @@ void timing_collect(Hierarchy &h);
 
 // multi-right-hand-side solves (batch_driver.cu)
 BatchWS &batch_workspace(Hierarchy &h, int K, cudaStream_t s);
-void batch_vcycle(Hierarchy &h, BatchWS &w, cudaStream_t s);
 void batch_iteration(Hierarchy &h, BatchWS &w, cudaStream_t s);  // async; scalars copied to w.h_d
 void batch_true_residual(Hierarchy &h, BatchWS &w, cudaStream_t s);  // async; tt copied to w.h_d
 void batch_push_flags(BatchWS &w, cudaStream_t s);

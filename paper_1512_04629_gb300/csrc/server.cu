@@ -197,7 +197,7 @@ int64_t batch_bytes(const Hierarchy &h, int K) {
     int64_t cyc = 0;
     for (int l = 0; l < h.nlev(); ++l) cyc += 4 * xb * (int64_t)h.lev[l]->n() * K;
     int64_t n0 = h.lev[0]->n();
-    int64_t pcg = 7 * 8 * n0 * K + (xb == 4 ? (h.nlev() == 1 ? 2 : 1) * 4 * n0 * K : 0);
+    int64_t pcg = 6 * 8 * n0 * K + xb * n0 * K + (xb == 4 ? 4 * n0 * K : 0);
     return cyc + pcg + (1 << 20);
 }
 
@@ -285,11 +285,8 @@ bool admit(amg_server *S, HState &H) {
             AMG_CUDA(cudaMemcpyAsync(H.dstage.ptr, H.hstage, sizeof(double) * H.n, cudaMemcpyHostToDevice, H.stream));
             src = H.dstage.as<double>();
         }
-        bat::scatter_column(H.n, w.K, c, src, w.B.as<double>(), H.stream);
-        bat::scatter_column(H.n, w.K, c, src, w.R.as<double>(), H.stream, w.R32.as<float>());
-        bat::zero_column(H.n, w.K, c, w.X.as<double>(), H.stream);
-        bat::zero_column(H.n, w.K, c, w.P.as<double>(), H.stream);
-        bat::zero_column(H.n, w.K, c, w.Q.as<double>(), H.stream);
+        bat::admit_column(H.n, w.K, c, src, w.B.as<double>(), w.R.as<double>(), w.R32.as<float>(), w.X.as<double>(),
+                          w.P.as<double>(), w.Q.as<double>(), H.stream);
         if (r->d_b) {
             stage_free(S, r, r->d_b, H.stream);  // after the scatters, in stream order
         } else {
