@@ -36,6 +36,28 @@ namespace {
 __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
+// The two halves, for kernels that load what no earlier kernel of the solve
+// writes -- the operator, its layout, its diagonal -- in between, so that
+// these loads overlap the kernel before.  Everything a solve kernel reads that
+// way is complete before its first launch: setup and re-sparsification end
+// with a stream synchronisation, and so does each layout built for a timed
+// trial.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// vectors written by the kernel before: coherent loads that stay behind the
+// dependency wait (a read-only load may be moved above it by the compiler)
+__device__ __forceinline__ double ld_dyn(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_dyn(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 
 static bool pdl_enabled() {
     static const bool on = [] {
@@ -240,19 +262,6 @@ __device__ __forceinline__ XT sell_row_sum(int32_t pos, int32_t row, const int32
 #endif
 constexpr int kPatBlocks = AMG_PAT_BLOCKS;  // resident blocks per SM the kernels are compiled for
 
-// vectors written by the kernel before: coherent loads that stay behind the
-// dependency wait (a read-only load may be moved above it by the compiler)
-__device__ __forceinline__ double ld_dyn(const double *p) {
-    double v;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float ld_dyn(const float *p) {
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
 // The table as the kernels hold it.  FP32 keeps an entry's value and offset
 // side by side, one 8-byte shared load per entry: two loads made the 27-point
 // residual load/store-bound (192^3: 94 -> 72 us).  FP64 keeps two arrays:
@@ -281,7 +290,7 @@ template <typename VT> struct PatSmem {
 // kernel's own predecessor has finished (the table does not depend on it)
 template <typename VT> __device__ __forceinline__ PatSmem<VT> pat_begin(const PatView<VT> &pt) {
     extern __shared__ __align__(16) unsigned char pat_raw[];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_launch_next();
     const int32_t ne = pt.npat * pt.width;
     VT *val = reinterpret_cast<VT *>(pat_raw);
     float2 *ent = reinterpret_cast<float2 *>(pat_raw);
@@ -302,7 +311,7 @@ template <typename VT> __device__ __forceinline__ PatSmem<VT> pat_begin(const Pa
         len[e] = __ldg(pt.len + e);
     }
     __syncthreads();
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     return PatSmem<VT>{val, delta, ent, dinv, len, pt.width};
 }
 
@@ -377,21 +386,102 @@ __device__ __forceinline__ void row_store(int32_t i, XT s, const XT *__restrict_
     }
 }
 
-template <typename VT, typename XT, int T, int OP>
+// the row's own operands of an operation, loaded before its sum is known
+template <typename XT> struct RowOwn {
+    XT b, d, x, o;
+};
+// what the kernel before may have written
+template <typename XT, int OP>
+__device__ __forceinline__ void own_dynamic(RowOwn<XT> &w, int32_t i, const XT *b, const XT *x, const XT *o1) {
+    if (kIsResid<OP>) w.b = ld_dyn(b + i);
+    if (OP == kPost) w.x = ld_dyn(x + i);
+    if (OP == kSpmvAdd) w.o = ld_dyn(o1 + i);
+}
+template <typename XT, int OP>
+__device__ __forceinline__ void own_store(const RowOwn<XT> &w, int32_t i, XT s, XT *o1, XT *o2) {
+    if (OP == kPost) {
+        o1[i] = w.x + w.d * s;
+    } else if (OP == kSpmv) {
+        o1[i] = s;
+    } else if (OP == kSpmvScale) {
+        o1[i] = s;
+        o2[i] = s * w.d;
+    } else if (OP == kResX) {
+        o2[i] = s;
+    } else {
+        o1[i] = w.o + s;
+    }
+}
+
+// Grids of at most kPreBlocks blocks per SM -- the small levels, whose kernels
+// are a chain of dependent loads and not work -- take a form that loads the
+// operator before it waits for the kernel before: the row bounds, the first
+// entries and the diagonal are then in registers when the vectors are ready,
+// and the chain that is left is one gather.  Larger grids run in several
+// waves, of which only the first could use it, and the registers would cost
+// them resident warps.
+constexpr int kPreBlocks = 4;
+static bool preload_grid(int blocks) { return blocks <= ::amg::resident_blocks(2048) * kPreBlocks; }
+
+template <typename VT, typename XT, int T, int OP, bool PRE>
 __global__ void __launch_bounds__(kThreads)
 csr_op_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const VT *__restrict__ v,
-              const XT *__restrict__ b, const XT *__restrict__ dinv, const XT *__restrict__ x,
-              XT *__restrict__ o1, XT *__restrict__ o2) {
-    pdl_begin();
+              const XT *b, const XT *dinv, const XT *x, XT *o1, XT *o2) {
+    constexpr bool SUB = kIsResid<OP>;
+    if constexpr (!PRE) pdl_begin();
+    else pdl_launch_next();
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int32_t i = (int32_t)(g / T);
     int t = (int)(g % T);
     int32_t p0 = 0, p1 = 0;
     if (i < n) { p0 = __ldg(rp + i); p1 = __ldg(rp + i + 1); }
-    const XT init = kIsResid<OP> && i < n && t == 0 ? b[i] : XT(0);
-    const XT s = csr_row_sum<VT, XT, T, kIsResid<OP>>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); }, init);
-    if (i >= n || t != 0) return;
-    row_store<XT, OP>(i, s, dinv, x, o1, o2);
+    const bool own = i < n && t == 0;
+    RowOwn<XT> w{};
+    if constexpr (!PRE) {
+        if (own && SUB) w.b = b[i];
+        const XT s = csr_row_sum<VT, XT, T, SUB>(p0, p1, t, ci, v, [&](int32_t j) { return __ldg(x + j); }, w.b);
+        if (!own) return;
+        if (OP == kPost || OP == kSpmvScale) w.d = dinv[i];
+        if (OP == kPost) w.x = x[i];
+        if (OP == kSpmvAdd) w.o = o1[i];
+        own_store<XT, OP>(w, i, s, o1, o2);
+    } else {
+        constexpr int V = Vec<VT>::V, NC = 2;  // chunks of the row held in registers
+        VT vv[NC][V];
+        int32_t cc[NC][V];
+        int32_t q = (p0 & ~(V - 1)) + t * V;
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (q + c * T * V < p1) Vec<VT>::load(v, ci, q + c * T * V, vv[c], cc[c]);
+        if (own && (OP == kPost || OP == kSpmvScale)) w.d = __ldg(dinv + i);
+        pdl_wait();
+        if (own) own_dynamic<XT, OP>(w, i, b, x, o1);
+        XT xv[NC][V];
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+                const int32_t e = q + c * T * V + u;
+                if (e >= p0 && e < p1) xv[c][u] = ld_dyn(x + cc[c][u]);
+            }
+        XT acc = own ? w.b : XT(0);
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+            for (int u = 0; u < V; ++u) {
+                const int32_t e = q + c * T * V + u;
+                if (e >= p0 && e < p1) acc = mac<SUB>(acc, cvt<VT, XT>(vv[c][u]), xv[c][u]);
+            }
+        for (q += NC * T * V; q < p1; q += T * V) {
+            Vec<VT>::load(v, ci, q, vv[0], cc[0]);
+#pragma unroll
+            for (int u = 0; u < V; ++u)
+                if (q + u < p1) acc = mac<SUB>(acc, cvt<VT, XT>(vv[0][u]), ld_dyn(x + cc[0][u]));
+        }
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o, T);
+        if (own) own_store<XT, OP>(w, i, acc, o1, o2);
+    }
 }
 
 // One lane per row of a SELL-32 operator; SHORT: every slice fits the
@@ -528,12 +618,13 @@ void part_op(const CycMat<double> &A, const double *b, const double *dinv, const
 // -- and the T parts are added by xor shuffles.  The row's sum therefore
 // runs in another order than a sequential one (not bit-equal to CSR).
 // CS: the operator's entries load with the evict-first policy.
-template <typename VT, typename XT, int OP, bool D16, int C, bool CS>
+template <typename VT, typename XT, int OP, bool D16, int C, bool CS, bool PRE>
 __global__ void __launch_bounds__(kThreads)
 sell_lanes_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ soff,
-                     const int32_t *__restrict__ sw, SellIdx ix, const VT *__restrict__ sv, const XT *__restrict__ b,
-                     const XT *__restrict__ dinv, const XT *__restrict__ x, XT *__restrict__ o1, XT *__restrict__ o2) {
-    pdl_begin();
+                     const int32_t *__restrict__ sw, SellIdx ix, const VT *__restrict__ sv, const XT *b,
+                     const XT *dinv, const XT *x, XT *o1, XT *o2) {
+    if constexpr (!PRE) pdl_begin();
+    else pdl_launch_next();
     constexpr int T = 32 / C, U = 4;
     const int32_t slice = (int32_t)(((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31, r = lane % C, t = lane / C;
@@ -542,8 +633,40 @@ sell_lanes_op_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t 
     const bool valid = pos < n;
     const int32_t i = valid ? (perm ? __ldg(perm + pos) : pos) : 0;
     const int32_t off = __ldg(soff + slice) + lane, w = __ldg(sw + slice);
-    auto gather = [&](int32_t j) { return __ldg(x + j); };
     constexpr bool SUB = kIsResid<OP>;
+    if constexpr (PRE) {  // see kPreBlocks: the lane's first H entries before the wait
+        constexpr int H = 8;
+        const int32_t nk = valid ? w / T : 0;
+        const bool own = valid && t == 0;
+        VT v[H];
+        int32_t c[H];
+#pragma unroll
+        for (int k = 0; k < H; ++k)
+            if (k < nk) {
+                v[k] = ld_ro<CS>(sv + off + k * 32);
+                c[k] = sell_col<D16, CS>(ix, off + k * 32, i);
+            }
+        RowOwn<XT> ro{};
+        if (own && (OP == kPost || OP == kSpmvScale)) ro.d = __ldg(dinv + i);
+        pdl_wait();
+        if (own) own_dynamic<XT, OP>(ro, i, b, x, o1);
+        XT acc = ro.b, xv[H];
+#pragma unroll
+        for (int k = 0; k < H; ++k)
+            if (k < nk) xv[k] = ld_dyn(x + c[k]);
+#pragma unroll
+        for (int k = 0; k < H; ++k)
+            if (k < nk) acc = mac<SUB>(acc, cvt<VT, XT>(v[k]), xv[k]);
+        auto dyn = [&](int32_t j) { return ld_dyn(x + j); };
+        int32_t k = H;
+        for (; k + U <= nk; k += U) acc = sell_short_sum<U, VT, XT, D16, CS, SUB>(acc, off + k * 32, i, ix, sv, dyn);
+        if (k < nk) acc = sell_short_any<VT, XT, D16, CS, SUB>(acc, nk - k, off + k * 32, i, ix, sv, dyn);
+#pragma unroll
+        for (int o = 16; o >= C; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (own) own_store<XT, OP>(ro, i, acc, o1, o2);
+        return;
+    }
+    auto gather = [&](int32_t j) { return __ldg(x + j); };
     XT acc = XT(0);
     if (valid) {
         if (SUB && t == 0) acc = b[i];
@@ -578,18 +701,22 @@ void launch_sell_lanes(const CycMat<VT> &A, const XT *b, const XT *dinv, const X
     const SellIdx ix{A.sci, A.sd};
     const int64_t warps = div_up((int64_t)n, (int64_t)C);
     const int g = (int)div_up(warps * 32, (int64_t)kThreads);
-    auto launch = [&](auto cs) {
-        constexpr bool CS = decltype(cs)::value;
+    auto launch = [&](auto cs, auto pre) {
+        constexpr bool CS = decltype(cs)::value, PRE = decltype(pre)::value;
         if (A.sd)
-            { pdl_launch(sell_lanes_op_kernel<VT, XT, OP, true, C, CS>, g, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, b, dinv, x, o1, o2); ::amg::count_launch(); }
+            { pdl_launch(sell_lanes_op_kernel<VT, XT, OP, true, C, CS, PRE>, g, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, b, dinv, x, o1, o2); ::amg::count_launch(); }
         else
-            { pdl_launch(sell_lanes_op_kernel<VT, XT, OP, false, C, CS>, g, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, b, dinv, x, o1, o2); ::amg::count_launch(); }
+            { pdl_launch(sell_lanes_op_kernel<VT, XT, OP, false, C, CS, PRE>, g, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, b, dinv, x, o1, o2); ::amg::count_launch(); }
     };
+    if (preload_grid(g)) {
+        launch(std::false_type(), std::true_type());
+        return;
+    }
     if constexpr (std::is_same<VT, double>::value && std::is_same<XT, double>::value) {
-        if (A.stream) launch(std::true_type());
-        else launch(std::false_type());
+        if (A.stream) launch(std::true_type(), std::false_type());
+        else launch(std::false_type(), std::false_type());
     } else {
-        launch(std::false_type());
+        launch(std::false_type(), std::false_type());
     }
 }
 
@@ -642,13 +769,19 @@ void dispatch_op(const CycMat<VT> &A, const XT *b, const XT *dinv, const XT *x, 
     } else {
         int T = threads_per_row(A.variant);
         int blocks = div_up((int64_t)n * T, kThreads);
+        auto launch = [&](auto tc) {
+            constexpr int L = decltype(tc)::value;
+            if (preload_grid(blocks)) pdl_launch(csr_op_kernel<VT, XT, L, OP, true>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2);
+            else pdl_launch(csr_op_kernel<VT, XT, L, OP, false>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2);
+            ::amg::count_launch();
+        };
         switch (T) {
-            case 1: { pdl_launch(csr_op_kernel<VT, XT, 1, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
-            case 2: { pdl_launch(csr_op_kernel<VT, XT, 2, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
-            case 4: { pdl_launch(csr_op_kernel<VT, XT, 4, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
-            case 8: { pdl_launch(csr_op_kernel<VT, XT, 8, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
-            case 16: { pdl_launch(csr_op_kernel<VT, XT, 16, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
-            default: { pdl_launch(csr_op_kernel<VT, XT, 32, OP>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, b, dinv, x, o1, o2); ::amg::count_launch(); } break;
+            case 1: launch(std::integral_constant<int, 1>{}); break;
+            case 2: launch(std::integral_constant<int, 2>{}); break;
+            case 4: launch(std::integral_constant<int, 4>{}); break;
+            case 8: launch(std::integral_constant<int, 8>{}); break;
+            case 16: launch(std::integral_constant<int, 16>{}); break;
+            default: launch(std::integral_constant<int, 32>{}); break;
         }
     }
     AMG_CHECK_LAUNCH();
@@ -1063,13 +1196,25 @@ __global__ void to_f32_scaled_kernel(int64_t n, const double *__restrict__ src, 
 // coarse solve: x = inv b, one warp per row
 // ---------------------------------------------------------------------------
 template <typename XT>
-__global__ void coarse_kernel(int32_t n, const double *__restrict__ inv, const XT *__restrict__ b, XT *__restrict__ x) {
-    pdl_begin();
+__global__ void coarse_kernel(int32_t n, const double *__restrict__ inv, const XT *b, XT *x) {
+    constexpr int H = 4;  // entries a lane loads before the wait: the whole row up to 128 unknowns
+    pdl_launch_next();
     int lane = threadIdx.x & 31;
     int32_t row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (row >= n) return;
+    const double *a = inv + (size_t)row * n;
+    double av[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) av[k] = lane + 32 * k < n ? __ldg(a + lane + 32 * k) : 0.0;
+    pdl_wait();
     double s = 0.0;
-    for (int32_t j = lane; j < n; j += 32) s += inv[(size_t)row * n + j] * (double)b[j];
+    XT bv[H];
+#pragma unroll
+    for (int k = 0; k < H; ++k) bv[k] = lane + 32 * k < n ? ld_dyn(b + lane + 32 * k) : XT(0);
+#pragma unroll
+    for (int k = 0; k < H; ++k)
+        if (32 * k < n) s += av[k] * (double)bv[k];
+    for (int32_t j = lane + 32 * H; j < n; j += 32) s += __ldg(a + j) * (double)ld_dyn(b + j);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) x[row] = (XT)s;
 }

@@ -500,6 +500,7 @@ template <typename VT, typename XT> static void autotune_level(Hierarchy &h, Lev
         V.variant = c;
         const int C = sell_height(c);
         if (C && V.sell_c != C) build_sell<VT>(V, s, C);
+        AMG_CUDA(cudaStreamSynchronize(s));  // cycle kernels may read their operator before their dependency wait
         CycMat<VT> m = op_mat<VT>(V);
         cyc::post_smooth<VT, XT>(m, V.x.as<XT>(), V.b.as<XT>(), dinv, V.xo.as<XT>(), s);  // warm-up
         float tmin = 1e30f;
@@ -687,6 +688,7 @@ template <typename XT> static bool autotune_transfers_at(Level &V, Level &C, cud
                 continue;
             if ((C == 16 && mean < 4.0) || (C == 8 && mean < 8.0)) continue;
             if (C && (!S.sv.ptr || S.c != C)) build_sell_copy<XT>(M, vals, S, s, C);
+            AMG_CUDA(cudaStreamSynchronize(s));  // as in autotune_level
             variant = v;
             run();
             float tmin = 1e30f;
