@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "cycle_ops.cuh"
+#include "fp_convert.cuh"
 
 namespace amg {
 namespace cyc {
@@ -929,12 +930,12 @@ static_assert(kThreads == 256, "two-level reduction assumes groups of 256 blocks
 // ---------------------------------------------------------------------------
 // PCG kernels (FP64)
 // ---------------------------------------------------------------------------
-__global__ void p_update_kernel(int32_t n, const double *__restrict__ z, double *__restrict__ p,
-                                const PcgScalars *sc) {
+template <typename ZT>
+__global__ void p_update_kernel(int32_t n, const ZT *__restrict__ z, double *__restrict__ p, const PcgScalars *sc) {
     pdl_begin();
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    p[i] = z[i] + sc->beta * p[i];
+    p[i] = widen(z[i]) + sc->beta * p[i];
 }
 
 // q = A p (SELL-32, one thread per row) and p . q; each warp walks slices
@@ -1013,8 +1014,7 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
 
 __global__ void __launch_bounds__(kThreads)
 xr_update_kernel(int32_t n, const double *__restrict__ p, const double *__restrict__ q, double *__restrict__ x,
-                 double *__restrict__ r, const PcgScalars *sc, Reduce red, const double *__restrict__ dinv0,
-                 double *__restrict__ x0, double *__restrict__ xs) {
+                 double *__restrict__ r, const PcgScalars *sc, Reduce red, CycleInput next, double *__restrict__ xs) {
     pdl_begin();
     block_partials_begin();
     const double alpha = sc->alpha;
@@ -1030,7 +1030,14 @@ xr_update_kernel(int32_t n, const double *__restrict__ p, const double *__restri
             ri -= alpha * q[i];
             r[i] = ri;
         }
-        if (x0) x0[i] = ri * dinv0[i];  // the next cycle's level-0 pre-smooth from zero
+        // the next cycle's input and its level-0 pre-smooth from zero
+        if (next.x64) {
+            next.x64[i] = ri * __ldg(next.dinv64 + i);
+        } else if (next.x32) {
+            const float r32 = narrow(ri);
+            next.r32[i] = r32;
+            next.x32[i] = r32 * __ldg(next.dinv32 + i);
+        }
         part[0] += ri * ri;
     }
     block_partials<1>(part, red);
@@ -1160,15 +1167,17 @@ post_rz_pat_kernel(int32_t n, PatView<double> pt, const double *x, const double 
     block_partials<ZQ ? 2 : 1>(part, red);
 }
 
+// r.z and z.q of the FP32 cycle's output, which stays in FP32 (the search
+// direction's update widens it again: 4 bytes a value instead of 8 written
+// and read)
 __global__ void __launch_bounds__(kThreads)
-to_f64_rz_kernel(int32_t n, const float *__restrict__ z32, double *__restrict__ z, const double *__restrict__ r,
-                 const double *__restrict__ q, PcgScalars *sc, Reduce red) {
+rz32_kernel(int32_t n, const float *__restrict__ z32, const double *__restrict__ r, const double *__restrict__ q,
+            PcgScalars *sc, Reduce red) {
     pdl_begin();
     block_partials_begin();
     double part[2] = {0.0, 0.0};
     for (int32_t i = blockIdx.x * kThreads + threadIdx.x; i < n; i += gridDim.x * kThreads) {
-        double zi = (double)z32[i];
-        z[i] = zi;
+        const double zi = widen(z32[i]);
         part[0] += r[i] * zi;
         part[1] += zi * q[i];
     }
@@ -1187,7 +1196,7 @@ __global__ void to_f32_scaled_kernel(int64_t n, const double *__restrict__ src, 
     pdl_begin();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    float v = (float)src[i];
+    const float v = narrow(src[i]);
     dst[i] = v;
     xdst[i] = v * d[i];
 }
@@ -1374,10 +1383,13 @@ void coarse_solve(int32_t n, const double *inv, const XT *b, XT *x, cudaStream_t
     AMG_CHECK_LAUNCH();
 }
 
-void pcg_p_update(int32_t n, const double *z, double *p, const PcgScalars *sc, cudaStream_t s) {
-    { pdl_launch(p_update_kernel, div_up(n, kThreads), kThreads, 0, s, n, z, p, sc); ::amg::count_launch(); }
+template <typename ZT> void pcg_p_update(int32_t n, const ZT *z, double *p, const PcgScalars *sc, cudaStream_t s) {
+    { pdl_launch(p_update_kernel<ZT>, div_up(n, kThreads), kThreads, 0, s, n, z, p, sc); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
 }
+
+template void pcg_p_update<double>(int32_t, const double *, double *, const PcgScalars *, cudaStream_t);
+template void pcg_p_update<float>(int32_t, const float *, double *, const PcgScalars *, cudaStream_t);
 
 template <int T>
 static void launch_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc, Reduce red, cudaStream_t s) {
@@ -1438,10 +1450,10 @@ void pcg_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc,
 }
 
 void pcg_xr_update(int32_t n, const double *p, const double *q, double *x, double *r, PcgScalars *sc,
-                   Reduce red, cudaGraphConditionalHandle handle, bool use_handle, const double *dinv0,
-                   double *x0, double *xs, cudaStream_t s) {
+                   Reduce red, cudaGraphConditionalHandle handle, bool use_handle, const CycleInput &next,
+                   double *xs, cudaStream_t s) {
     int blocks = reduce_blocks(n);
-    { pdl_launch(xr_update_kernel, blocks, kThreads, 0, s, n, p, q, x, r, sc, red, dinv0, x0, xs); ::amg::count_launch(); }
+    { pdl_launch(xr_update_kernel, blocks, kThreads, 0, s, n, p, q, x, r, sc, red, next, xs); ::amg::count_launch(); }
     launch_finish<1, kFinXr>(blocks, red, sc, s, handle, use_handle);
     AMG_CHECK_LAUNCH();
 }
@@ -1499,10 +1511,10 @@ bool post_smooth_rz(const CycMat<double> &A, const double *x, const double *b, c
     return true;
 }
 
-void to_f64_rz(int32_t n, const float *z32, double *z, const double *r, const double *q, PcgScalars *sc, Reduce red,
-               cudaStream_t s) {
+void pcg_rz32(int32_t n, const float *z32, const double *r, const double *q, PcgScalars *sc, Reduce red,
+              cudaStream_t s) {
     int blocks = reduce_blocks(n);
-    { pdl_launch(to_f64_rz_kernel, blocks, kThreads, 0, s, n, z32, z, r, q, sc, red); ::amg::count_launch(); }
+    { pdl_launch(rz32_kernel, blocks, kThreads, 0, s, n, z32, r, q, sc, red); ::amg::count_launch(); }
     launch_finish<2, kFinRz>(blocks, red, sc, s);
     AMG_CHECK_LAUNCH();
 }

@@ -96,6 +96,15 @@ struct Reduce {
 };
 constexpr int kMaxReduceBlocks = 65536;
 
+// What the x, r update writes for the next cycle: its level-0 pre-smooth
+// x = D_0^-1 r, in FP32 modes with the FP32 residual (null: nothing).
+struct CycleInput {
+    const double *dinv64 = nullptr;
+    double *x64 = nullptr;
+    const float *dinv32 = nullptr;
+    float *r32 = nullptr, *x32 = nullptr;
+};
+
 namespace cyc {
 
 int threads_per_row(int variant);
@@ -117,23 +126,23 @@ template <typename XT>
 void coarse_solve(int32_t n, const double *inv, const XT *b, XT *x, cudaStream_t s);
 
 // PCG (FP64)
-void pcg_p_update(int32_t n, const double *z, double *p, const PcgScalars *sc, cudaStream_t s);
+template <typename ZT> void pcg_p_update(int32_t n, const ZT *z, double *p, const PcgScalars *sc, cudaStream_t s);
 void pcg_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc, Reduce red, cudaStream_t s);
 // x += alpha p, r -= alpha q, rr, its += 1; with a graph handle, the WHILE
 // condition is set to continue while rr > thresh2, its < max_its, no
 // breakdown and no divergence.  With the divergence test on (sc->divf > 0),
 // a step that starts a window first copies x to xs.
 void pcg_xr_update(int32_t n, const double *p, const double *q, double *x, double *r, PcgScalars *sc,
-                   Reduce red, cudaGraphConditionalHandle handle, bool use_handle, const double *dinv0,
-                   double *x0, double *xs, cudaStream_t s);
+                   Reduce red, cudaGraphConditionalHandle handle, bool use_handle, const CycleInput &next,
+                   double *xs, cudaStream_t s);
 // level-0 post-smoothing that also forms rho = r.z and, when q is given
 // (flexible CG), z.q, and beta: z is the output, r = b the cycle input.
 // Returns false (nothing launched) for an empty level.
 bool post_smooth_rz(const CycMat<double> &A, const double *x, const double *b, const double *dinv, double *z,
                     const double *q, PcgScalars *sc, Reduce red, cudaStream_t s);
-// z = (double) z32 and rho = r.z, z.q (FP32 cycles)
-void to_f64_rz(int32_t n, const float *z32, double *z, const double *r, const double *q, PcgScalars *sc, Reduce red,
-               cudaStream_t s);
+// rho = r.z and z.q with the FP32 cycle's output as it is
+void pcg_rz32(int32_t n, const float *z32, const double *r, const double *q, PcgScalars *sc, Reduce red,
+              cudaStream_t s);
 // out = a .* d (pre-smooth from zero)
 template <typename XT> void scale(int64_t n, const XT *a, const XT *d, XT *out, cudaStream_t s);
 // dst = (float) src and xdst = dst .* d (FP32 cycle input with its pre-smooth)

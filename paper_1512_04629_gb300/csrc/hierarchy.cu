@@ -1174,17 +1174,17 @@ bool vcycle_f64(Hierarchy &h, const double *r, double *z, cudaStream_t s, const 
     int64_t n = h.lev[0]->n();
     Level &V0 = *h.lev[0];
     CycleCtl c32 = ctl;
-    if (h.nlev() > 1) {
+    if (h.nlev() == 1) {
+        cyc::convert_vec_from_f64<float>(r, h.r32.as<float>(), n, s);
+    } else if (!ctl.x0_ready) {
         // FP32 input and its level-0 pre-smooth in one pass
         cyc::to_f32_scaled(n, r, V0.dinv32.as<float>(), h.r32.as<float>(), V0.x.as<float>(), s);
         c32.x0_ready = true;
-    } else {
-        cyc::convert_vec_from_f64<float>(r, h.r32.as<float>(), n, s);
     }
     vcycle_impl<float>(h, h.r32.as<float>(), h.z32.as<float>(), s, c32);
-    if (ctl.fuse_rz) {
-        timed(h, 6, 0, 28.0 * n, s, [&] {
-            cyc::to_f64_rz((int32_t)n, h.z32.as<float>(), z, r, ctl.q, h.dscal(), h.reduce(), s);
+    if (ctl.fuse_rz) {  // the output stays in h.z32
+        timed(h, 6, 0, 20.0 * n, s, [&] {
+            cyc::pcg_rz32((int32_t)n, h.z32.as<float>(), r, ctl.q, h.dscal(), h.reduce(), s);
         });
         return true;
     }
@@ -1206,6 +1206,7 @@ namespace {
 struct Run {
     int steps = 0, replacements = 0;
     bool converged = false, breakdown = false, diverged = false;
+    bool exact = false;  // rnorm is the true residual norm of x as it is
     double rnorm = 0.0;
 };
 
@@ -1253,25 +1254,27 @@ double true_resnorm(Hierarchy &h, const double *b, const double *x, cudaStream_t
     return std::sqrt(h.h_scal->tt);
 }
 
-// In FP64 the level-0 pre-smooth x0 = D0^-1 r of the next cycle is written by
-// the x, r update; after r is set any other way it is formed here.
+// The level-0 pre-smooth x0 = D0^-1 r of the next cycle (and its FP32 input) is
+// written by the x, r update; after r is set any other way it is formed here.
 void refresh_x0(Hierarchy &h, cudaStream_t s) {
-    if (h.opt.precision != AMG_PREC_FP64 || h.nlev() < 2) return;
+    if (h.nlev() < 2) return;
     Level &V0 = *h.lev[0];
-    cyc::scale<double>(V0.n(), h.pr.as<double>(), V0.dinv.as<double>(), V0.x.as<double>(), s);
+    if (h.opt.precision == AMG_PREC_FP64)
+        cyc::scale<double>(V0.n(), h.pr.as<double>(), V0.dinv.as<double>(), V0.x.as<double>(), s);
+    else
+        cyc::to_f32_scaled(V0.n(), h.pr.as<double>(), V0.dinv32.as<float>(), h.r32.as<float>(), V0.x.as<float>(), s);
 }
 
-// r = b - A x, p = 0, start = 1 (the next body sets beta = 0); returns ||r||
-double pcg_start(Hierarchy &h, const double *b, const double *x, cudaStream_t s) {
+// r = t, the true residual just formed (h.pt), p = 0, start = 1 (the next body
+// sets beta = 0)
+void pcg_start(Hierarchy &h, cudaStream_t s) {
     int64_t n = h.lev[0]->n();
-    double rn = true_resnorm(h, b, x, s);
     AMG_CUDA(cudaMemcpyAsync(h.pr.ptr, h.pt.ptr, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     refresh_x0(h, s);
     AMG_CUDA(cudaMemsetAsync(h.pp.ptr, 0, sizeof(double) * n, s));
     h.h_scal->start = 1;
     h.h_scal->breakdown = 0;
     write_scalars(h, s);
-    return rn;
 }
 
 // one CG step on the internal x (h.px)
@@ -1288,14 +1291,25 @@ void pcg_body(Hierarchy &h, cudaStream_t s, cudaGraphConditionalHandle handle, b
         timed(h, 6, 0, 24.0 * n, s, [&] {
             cyc::pcg_rz(n, h.pr.as<double>(), h.pz.as<double>(), h.pq.as<double>(), h.dscal(), h.reduce(), s);
         });
-    timed(h, 6, 0, 24.0 * n, s, [&] { cyc::pcg_p_update(n, h.pz.as<double>(), h.pp.as<double>(), h.dscal(), s); });
+    const bool fp64 = h.opt.precision == AMG_PREC_FP64;
+    timed(h, 6, 0, fp64 ? 24.0 * n : 20.0 * n, s, [&] {
+        if (fp64) cyc::pcg_p_update(n, h.pz.as<double>(), h.pp.as<double>(), h.dscal(), s);
+        else cyc::pcg_p_update(n, h.z32.as<float>(), h.pp.as<double>(), h.dscal(), s);
+    });
     timed(h, 5, 0, ap_bytes, s, [&] { cyc::pcg_ap(A0, h.pp.as<double>(), h.pq.as<double>(), h.dscal(), h.reduce(), s); });
-    bool fp64 = h.opt.precision == AMG_PREC_FP64 && h.nlev() > 1;
     Level &V0 = *h.lev[0];
-    timed(h, 6, 0, fp64 ? 64.0 * n : 48.0 * n, s, [&] {
+    CycleInput next;
+    if (h.nlev() > 1 && fp64) {
+        next.dinv64 = V0.dinv.as<double>();
+        next.x64 = V0.x.as<double>();
+    } else if (h.nlev() > 1) {
+        next.dinv32 = V0.dinv32.as<float>();
+        next.r32 = h.r32.as<float>();
+        next.x32 = V0.x.as<float>();
+    }
+    timed(h, 6, 0, 48.0 * n + (next.x64 ? 16.0 * n : next.x32 ? 12.0 * n : 0.0), s, [&] {
         cyc::pcg_xr_update(n, h.pp.as<double>(), h.pq.as<double>(), h.px.as<double>(), h.pr.as<double>(), h.dscal(),
-                           h.reduce(), handle, use_handle, fp64 ? V0.dinv.as<double>() : nullptr,
-                           fp64 ? V0.x.as<double>() : nullptr, h.pxs.as<double>(), s);
+                           h.reduce(), handle, use_handle, next, h.pxs.as<double>(), s);
     });
 }
 
@@ -1396,7 +1410,10 @@ void pcg_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int ma
         if (sc.rr > thresh2) return;  // step budget used up
         double tn = true_resnorm(h, b, h.px.as<double>(), s);
         run.rnorm = tn;
-        if (tn <= tol * bnorm) { run.converged = true; return; }
+        if (tn <= tol * bnorm) {
+            run.converged = run.exact = true;
+            return;
+        }
         AMG_CUDA(cudaMemcpyAsync(h.pr.ptr, h.pt.ptr, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
         refresh_x0(h, s);
         run.replacements++;
@@ -1415,6 +1432,7 @@ void pcg_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int ma
 struct GmRun {
     int steps = 0, replacements = 0;
     bool converged = false, breakdown = false;
+    bool exact = false;  // rnorm is the true residual norm of x as it is
     double rnorm = 0.0;
 };
 
@@ -1510,10 +1528,11 @@ void gm_ensure_graph(Hierarchy &h) {
 }
 
 // new cycle from the internal x (h.px): r = b - A x, v_0 = r / ||r||,
-// g = ||r|| e_1, x0 = x; returns ||r||
-double gm_start(Hierarchy &h, const double *b, double thresh, cudaStream_t s) {
+// g = ||r|| e_1, x0 = x; returns ||r|| (`known`: it, when the true residual of
+// x has just been formed and is still in h.pt)
+double gm_start(Hierarchy &h, const double *b, double thresh, cudaStream_t s, double known = -1.0) {
     const int64_t n = h.lev[0]->n();
-    double rn = true_resnorm(h, b, h.px.as<double>(), s);
+    const double rn = known >= 0.0 ? known : true_resnorm(h, b, h.px.as<double>(), s);
     AMG_CUDA(cudaMemcpyAsync(h.gx0.ptr, h.px.ptr, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     GmresScalars &c = *h.h_gsc;
     c.m = h.gm_m;
@@ -1573,24 +1592,29 @@ void gm_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int max
             gm_form_x(h, s);
             const double tn = gm_start(h, b, thresh, s);
             run.rnorm = tn;
-            if (tn <= thresh) { run.converged = true; return; }
+            if (tn <= thresh) {
+                run.converged = run.exact = true;
+                return;
+            }
             run.replacements++;
         }
     }
     gm_form_x(h, s);
 }
 
+// fin: receives the true residual norm of the final x when it is known
 amg_status solve_gmres(Hierarchy &h, const double *b, double bnorm, double tol, int max_it, bool adaptive,
-                       cudaStream_t s, amg_solve_info *info) {
+                       cudaStream_t s, amg_solve_info *info, double *fin) {
     gm_workspace(h, s);
     const int64_t n = h.lev[0]->n();
     double *x = h.px.as<double>();
     const double thresh = tol * bnorm;
     h.h_gsc->its = 0;
     if (!adaptive) {
-        const double r0 = gm_start(h, b, thresh, s);
+        const double r0 = gm_start(h, b, thresh, s, bnorm);  // x = 0: the residual that gave ||b||
         GmRun run;
         gm_iterate(h, b, bnorm, tol, max_it, s, run);
+        if (run.exact) *fin = run.rnorm;
         info->iterations = run.steps;
         info->replacements = run.replacements;
         info->conv_factor = run.steps > 0 ? std::pow(run.rnorm / r0, 1.0 / run.steps) : 0.0;
@@ -1602,7 +1626,7 @@ amg_status solve_gmres(Hierarchy &h, const double *b, double bnorm, double tol, 
     const int k = std::max(1, h.opt.k_check), sl = std::max(1, h.opt.s_levels);
     TmpBuf xs(sizeof(double) * (n + kPad), s);
     double rstart = bnorm;
-    gm_start(h, b, thresh, s);
+    gm_start(h, b, thresh, s, bnorm);
     int total = 0;
     bool converged = false, breakdown = false;
     while (total < max_it) {
@@ -1611,8 +1635,12 @@ amg_status solve_gmres(Hierarchy &h, const double *b, double bnorm, double tol, 
         gm_iterate(h, b, bnorm, tol, std::min(k, max_it - total), s, run);
         total += run.steps;
         info->replacements += run.replacements;
-        double rend = true_resnorm(h, b, x, s);
-        if (run.converged || rend <= thresh) { converged = true; break; }
+        double rend = run.exact ? run.rnorm : true_resnorm(h, b, x, s);
+        if (run.converged || rend <= thresh) {
+            converged = true;
+            *fin = rend;
+            break;
+        }
         breakdown = run.breakdown;
         const double factor = run.steps > 0 ? std::pow(rend / rstart, 1.0 / run.steps) : 1.0;
         if (factor > h.opt.rho_max || breakdown) {
@@ -1629,7 +1657,7 @@ amg_status solve_gmres(Hierarchy &h, const double *b, double bnorm, double tol, 
                     AMG_CUDA(cudaMemcpyAsync(x, xs.ptr, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
                     rend = rstart;
                 }
-                gm_start(h, b, thresh, s);
+                gm_start(h, b, thresh, s, back ? -1.0 : rend);
             }
         }
         rstart = rend;
@@ -1652,14 +1680,17 @@ amg_status solve(Hierarchy &h, const double *b, double *x_out, double tol, int m
     double bnorm = true_resnorm(h, b, x, s);
     if (!std::isfinite(bnorm)) throw Error(AMG_ERR_INVALID, "b has a non-finite value");
     amg_status st = AMG_OK;
+    double fin = -1.0;  // the true residual norm of the final x, when a check has just formed it
     if (bnorm == 0.0) {
         info->status = AMG_OK;
     } else if (h.opt.krylov == AMG_KRYLOV_GMRES) {
-        st = solve_gmres(h, b, bnorm, tol, max_it, adaptive, s, info);
+        st = solve_gmres(h, b, bnorm, tol, max_it, adaptive, s, info, &fin);
     } else if (!adaptive) {
-        double r0 = pcg_start(h, b, x, s);
+        const double r0 = bnorm;  // x = 0: the residual that gave ||b||
+        pcg_start(h, s);
         Run run;
         pcg_iterate(h, b, bnorm, tol, max_it, r0, h.opt.div_factor, s, run);
+        if (run.exact) fin = run.rnorm;
         info->iterations = run.steps;
         info->replacements = run.replacements;
         info->conv_factor = run.steps > 0 ? std::pow(run.rnorm / r0, 1.0 / run.steps) : 0.0;
@@ -1671,7 +1702,8 @@ amg_status solve(Hierarchy &h, const double *b, double *x_out, double tol, int m
         int k = std::max(1, h.opt.k_check), sl = std::max(1, h.opt.s_levels);
         TmpBuf xs(sizeof(double) * (n + kPad), s);
         double rstart = bnorm;
-        double rnow = pcg_start(h, b, x, s);
+        double rnow = bnorm;  // x = 0: the residual that gave ||b||
+        pcg_start(h, s);
         int total = 0;
         bool converged = false, breakdown = false, diverged = false;
         const double divf = h.opt.div_factor;
@@ -1681,8 +1713,12 @@ amg_status solve(Hierarchy &h, const double *b, double *x_out, double tol, int m
             pcg_iterate(h, b, bnorm, tol, std::min(k, max_it - total), rnow, 0.0, s, run);
             total += run.steps;
             info->replacements += run.replacements;
-            double rend = true_resnorm(h, b, x, s);
-            if (run.converged || rend <= tol * bnorm) { converged = true; break; }
+            double rend = run.exact ? run.rnorm : true_resnorm(h, b, x, s);
+            if (run.converged || rend <= tol * bnorm) {
+                converged = true;
+                fin = rend;
+                break;
+            }
             breakdown = run.breakdown;
             rnow = run.rnorm;
             double factor = run.steps > 0 ? std::pow(rend / rstart, 1.0 / run.steps) : 1.0;
@@ -1709,7 +1745,8 @@ amg_status solve(Hierarchy &h, const double *b, double *x_out, double tol, int m
                         AMG_CUDA(cudaMemcpyAsync(x, xs.ptr, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
                         rend = rstart;
                     }
-                    rnow = pcg_start(h, b, x, s);
+                    rnow = back ? true_resnorm(h, b, x, s) : rend;
+                    pcg_start(h, s);
                 }
             }
             rstart = rend;
@@ -1718,7 +1755,7 @@ amg_status solve(Hierarchy &h, const double *b, double *x_out, double tol, int m
         st = converged ? AMG_OK : diverged ? AMG_DIVERGED : (breakdown ? AMG_BREAKDOWN : AMG_NOT_CONVERGED);
     }
     if (bnorm > 0.0) {
-        double fin = true_resnorm(h, b, x, s);
+        if (fin < 0.0) fin = true_resnorm(h, b, x, s);
         info->final_relres = fin / bnorm;
         if (adaptive) info->conv_factor = info->iterations > 0 ? std::pow(info->final_relres, 1.0 / info->iterations) : 0.0;
     }
