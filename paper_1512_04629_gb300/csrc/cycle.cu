@@ -22,70 +22,12 @@
 #include "common.cuh"
 #include "cycle_ops.cuh"
 #include "fp_convert.cuh"
+#include "pdl.cuh"
 
 namespace amg {
 namespace cyc {
 
 namespace {
-
-// Programmatic dependent launch: the solve-path kernels go out with the
-// stream-serialisation attribute, so the next kernel's blocks are scheduled
-// while the current one runs (its launch latency is hidden), and every such
-// kernel begins with pdl_begin(): it lets its own dependent launch, then
-// waits until the kernel before it has completed and its writes are visible.
-// Without the attribute (or with AMG_PDL=0) both instructions do nothing.
-__device__ __forceinline__ void pdl_begin() {
-    asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
-}
-// The two halves, for kernels that load what no earlier kernel of the solve
-// writes -- the operator, its layout, its diagonal -- in between, so that
-// these loads overlap the kernel before.  Everything a solve kernel reads that
-// way is complete before its first launch: setup and re-sparsification end
-// with a stream synchronisation, and so does each layout built for a timed
-// trial.
-__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// vectors written by the kernel before: coherent loads that stay behind the
-// dependency wait (a read-only load may be moved above it by the compiler)
-__device__ __forceinline__ double ld_dyn(const double *p) {
-    double v;
-    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
-    return v;
-}
-__device__ __forceinline__ float ld_dyn(const float *p) {
-    float v;
-    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
-
-static bool pdl_enabled() {
-    static const bool on = [] {
-        const char *e = std::getenv("AMG_PDL");
-        return !(e && e[0] == '0');
-    }();
-    return on;
-}
-
-template <typename... KArgs, typename... Args>
-static void pdl_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
-    if (!pdl_enabled()) {
-        kern<<<grid, block, smem, s>>>(std::forward<Args>(args)...);
-        return;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    AMG_CUDA(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
-}
 
 constexpr int kThreads = 256;
 
@@ -791,54 +733,18 @@ void dispatch_op(const CycMat<VT> &A, const XT *b, const XT *dinv, const XT *x, 
 // ---------------------------------------------------------------------------
 // deterministic block reduction with last-block finish
 // ---------------------------------------------------------------------------
-// Block partials without a block-wide barrier at the end: every thread parks
-// its values in shared memory; the last warp of the block to arrive (a shared
-// arrival counter, zeroed when the kernel starts) adds them, lane l the
-// values l, l + 32, ... in warp order and then the 32 sums by shuffles, and
-// stores the block partial.  Warps that finish early leave at once instead of
-// waiting for the block's slowest gathers.  A shuffle tree in every warp
-// would issue 40 FP64 warp instructions a block where this issues 12; with
-// eight resident blocks per SM, all ending together, that is 2 us of the FP64
-// pipe at the end of each reducing kernel.  A one-block finisher kernel
-// launched next sums the block partials in block order: no atomics on
-// floating-point values, no fences on the producers' critical path, a
-// deterministic result.
-__device__ __forceinline__ unsigned *arrival_counter() {
-    __shared__ unsigned c;
-    return &c;
-}
-
-// every kernel that calls block_partials calls this first (all threads)
-__device__ __forceinline__ void block_partials_begin() {
-    if (threadIdx.x == 0) *arrival_counter() = 0u;
-    __syncthreads();
-}
-
-template <int NV>
-__device__ __forceinline__ void block_partials(double (&v)[NV], Reduce red) {
-    __shared__ double sh[NV][kThreads];
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k];
-    __threadfence_block();
-    __syncwarp();
-    unsigned ticket = 0;
-    if (lane == 0) ticket = atomicAdd(arrival_counter(), 1u);
-    if (__shfl_sync(0xffffffffu, ticket, 0) != kThreads / 32 - 1) return;
-    __threadfence_block();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        double t = ((volatile double *)sh[k])[lane];
-#pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) t += ((volatile double *)sh[k])[lane + 32 * w];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) red.partials[k * kMaxReduceBlocks + blockIdx.x] = t;
-    }
-}
-
 enum Fin { kFinAp = 0, kFinXr = 1, kFinRz = 2, kFinTt = 3 };
 
 constexpr int kFinThreads = 1024;
+
+// what the last step of a reduction needs besides the sums: the WHILE
+// condition of the captured loop for the x, r update, and whether the reducing
+// kernel finishes itself
+struct FinCtl {
+    cudaGraphConditionalHandle handle{};
+    int use_handle = 0;
+    int fused = 0;
+};
 
 // finish of r.z / z.q: beta and rho (start: beta = 0)
 __device__ __forceinline__ void finish_rz(PcgScalars *sc, double rz, double zq) {
@@ -852,9 +758,107 @@ __device__ __forceinline__ void finish_rz(PcgScalars *sc, double rz, double zq) 
     sc->start = 0;
 }
 
+// the CG scalars from the finished sums (one thread)
+template <int NV, int FIN>
+__device__ __forceinline__ void finish_scalars(const double (&t)[NV], PcgScalars *sc, const FinCtl &ctl) {
+    if (FIN == kFinAp) {
+        sc->pq = t[0];
+        bool ok = t[0] > 0.0 && sc->rho > 0.0;
+        if (!ok) sc->breakdown = 1;
+        sc->alpha = ok ? sc->rho / t[0] : 0.0;
+    } else if (FIN == kFinXr) {
+        sc->rr = t[0];
+        int its = sc->its + 1;
+        sc->its = its;
+        if (sc->divf > 0.0 && !sc->breakdown) {
+            // the window test, in the oracle's form: norms, not squares
+            const double rn = sqrt(t[0]);
+            const bool end = its % sc->kwin == 0;
+            if (!isfinite(rn) || (end && rn > sc->divf * sc->rn_ws)) sc->diverged = 1;
+            else if (end) sc->rn_ws = rn;
+        }
+        if (ctl.use_handle) {
+            bool go = t[0] > sc->thresh2 && its < sc->max_its && !sc->breakdown && !sc->diverged && isfinite(t[0]);
+            cudaGraphSetConditional(ctl.handle, go ? 1u : 0u);
+        }
+    } else if (FIN == kFinRz) {
+        finish_rz(sc, t[0], NV > 1 ? t[NV - 1] : 0.0);
+    } else {
+        sc->tt = t[0];
+    }
+}
+
+// Reductions without a block-wide barrier at the end: every thread parks its
+// values in shared memory; the last warp of the block to arrive (a shared
+// arrival counter, zeroed when the kernel starts) adds them, lane l the
+// values l, l + 32, ... in warp order and then the 32 sums by shuffles, and
+// stores the block partial.  Warps that finish early leave at once instead of
+// waiting for the block's slowest gathers.  A shuffle tree in every warp
+// would issue 40 FP64 warp instructions a block where this issues 12; with
+// eight resident blocks per SM, all ending together, that is 2 us of the FP64
+// pipe at the end of each reducing kernel.
+//
+// The block partials are summed in a fixed order -- no atomics on floating-
+// point values, a deterministic result -- by the last block to finish on
+// grids of at most kFuseBlocks blocks (one warp, a few partials a lane; the
+// order does not depend on which block it is), and by a one-block finisher
+// kernel launched next on larger ones: there the single warp's rounds of
+// loads and the fence of every block cost what the launch saves.
+__device__ __forceinline__ unsigned *arrival_counter() {
+    __shared__ unsigned c;
+    return &c;
+}
+
+// every kernel that calls block_partials calls this first (all threads)
+__device__ __forceinline__ void block_partials_begin() {
+    if (threadIdx.x == 0) *arrival_counter() = 0u;
+    __syncthreads();
+}
+
+template <int NV, int FIN>
+__device__ __forceinline__ void block_partials(double (&v)[NV], Reduce red, PcgScalars *sc, const FinCtl &ctl) {
+    __shared__ double sh[NV][kThreads];
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sh[k][threadIdx.x] = v[k];
+    __threadfence_block();
+    __syncwarp();
+    unsigned ticket = 0;
+    if (lane == 0) ticket = atomicAdd(arrival_counter(), 1u);
+    if (__shfl_sync(0xffffffffu, ticket, 0) != kThreads / 32 - 1) return;
+    __threadfence_block();
+    double t[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        t[k] = ((volatile double *)sh[k])[lane];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) t[k] += ((volatile double *)sh[k])[lane + 32 * w];
+        for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        if (lane == 0) red.partials[k * kMaxReduceBlocks + blockIdx.x] = t[k];
+    }
+    if (!ctl.fused) return;
+    if (gridDim.x > 1) {
+        if (lane == 0) {
+            __threadfence();
+            ticket = atomicAdd(red.counter, 1u);
+        }
+        if (__shfl_sync(0xffffffffu, ticket, 0) != gridDim.x - 1) return;
+        __threadfence();
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            t[k] = 0.0;
+#pragma unroll 8
+            for (unsigned b = lane; b < gridDim.x; b += 32) t[k] += __ldcg(red.partials + k * kMaxReduceBlocks + b);
+            for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        }
+        if (lane == 0) *red.counter = 0u;
+    }
+    if (lane == 0) finish_scalars<NV, FIN>(t, sc, ctl);
+}
+
 template <int NV, int FIN>
 __global__ void __launch_bounds__(kFinThreads)
-finish_kernel(int nblocks, Reduce red, PcgScalars *sc, cudaGraphConditionalHandle handle, int use_handle) {
+finish_kernel(int nblocks, Reduce red, PcgScalars *sc, FinCtl ctl) {
     pdl_begin();
     __shared__ double sh[NV][kFinThreads / 32];
     double t[NV];
@@ -880,38 +884,29 @@ finish_kernel(int nblocks, Reduce red, PcgScalars *sc, cudaGraphConditionalHandl
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         t[k] = x;
     }
-    if (lane != 0) return;
-    if (FIN == kFinAp) {
-        sc->pq = t[0];
-        bool ok = t[0] > 0.0 && sc->rho > 0.0;
-        if (!ok) sc->breakdown = 1;
-        sc->alpha = ok ? sc->rho / t[0] : 0.0;
-    } else if (FIN == kFinXr) {
-        sc->rr = t[0];
-        int its = sc->its + 1;
-        sc->its = its;
-        if (sc->divf > 0.0 && !sc->breakdown) {
-            // the window test, in the oracle's form: norms, not squares
-            const double rn = sqrt(t[0]);
-            const bool end = its % sc->kwin == 0;
-            if (!isfinite(rn) || (end && rn > sc->divf * sc->rn_ws)) sc->diverged = 1;
-            else if (end) sc->rn_ws = rn;
-        }
-        if (use_handle) {
-            bool go = t[0] > sc->thresh2 && its < sc->max_its && !sc->breakdown && !sc->diverged && isfinite(t[0]);
-            cudaGraphSetConditional(handle, go ? 1u : 0u);
-        }
-    } else if (FIN == kFinRz) {
-        finish_rz(sc, t[0], NV > 1 ? t[NV - 1] : 0.0);
-    } else {
-        sc->tt = t[0];
-    }
+    if (lane == 0) finish_scalars<NV, FIN>(t, sc, ctl);
 }
 
+// 16 blocks (64 x 64): the solve 974 -> 948 us with its three reductions a step
+// finishing themselves; 400 to 600 blocks measure the same either way, and at
+// 900 to 1200 (all of 101^3 and 128^3) the finisher kernel is 1-5% of the
+// solve faster.
+constexpr int kFuseBlocks = 128;
+
+// how a reducing kernel of `blocks` blocks finishes
+FinCtl fin_ctl(int blocks, cudaGraphConditionalHandle handle = cudaGraphConditionalHandle{}, bool use_handle = false) {
+    FinCtl c;
+    c.handle = handle;
+    c.use_handle = use_handle ? 1 : 0;
+    c.fused = blocks <= kFuseBlocks;
+    return c;
+}
+
+// after the reducing kernel: the finisher where it does not finish itself
 template <int NV, int FIN>
-void launch_finish(int nblocks, Reduce red, PcgScalars *sc, cudaStream_t s,
-                   cudaGraphConditionalHandle handle = cudaGraphConditionalHandle{}, bool use_handle = false) {
-    { pdl_launch(finish_kernel<NV, FIN>, 1, kFinThreads, 0, s, nblocks, red, sc, handle, use_handle ? 1 : 0); ::amg::count_launch(); }
+void launch_finish(int nblocks, Reduce red, PcgScalars *sc, cudaStream_t s, const FinCtl &ctl) {
+    if (ctl.fused) return;
+    { pdl_launch(finish_kernel<NV, FIN>, 1, kFinThreads, 0, s, nblocks, red, sc, ctl); ::amg::count_launch(); }
 }
 
 // Grid of a reducing kernel: at most one resident wave, so every thread
@@ -945,7 +940,7 @@ template <bool D16, bool SHORT, bool RESID>
 __global__ void __launch_bounds__(kThreads)
 ap_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ soff, const int32_t *__restrict__ sw,
                SellIdx ix, const double *__restrict__ sv, const double *__restrict__ p, const double *__restrict__ b,
-               double *__restrict__ q, PcgScalars *sc, Reduce red) {
+               double *__restrict__ q, PcgScalars *sc, Reduce red, FinCtl ctl) {
     pdl_begin();
     block_partials_begin();
     double part[1] = {0.0};
@@ -964,13 +959,14 @@ ap_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__res
             part[0] += p[i] * s;
         }
     }
-    block_partials<1>(part, red);
+    block_partials<1, RESID ? kFinTt : kFinAp>(part, red, sc, ctl);
 }
 
 // the same with the operator stored by row patterns
 template <bool RESID>
 __global__ void __launch_bounds__(kThreads, kPatBlocks)
-ap_pat_kernel(int32_t n, PatView<double> pt, const double *p, const double *b, double *q, PcgScalars *sc, Reduce red) {
+ap_pat_kernel(int32_t n, PatView<double> pt, const double *p, const double *b, double *q, PcgScalars *sc, Reduce red,
+              FinCtl ctl) {
     block_partials_begin();
     const PatSmem<double> t = pat_begin(pt);
     double part[1] = {0.0};
@@ -981,14 +977,15 @@ ap_pat_kernel(int32_t n, PatView<double> pt, const double *p, const double *b, d
         q[i] = s;
         part[0] += RESID ? s * s : pi * s;
     });
-    block_partials<1>(part, red);
+    block_partials<1, RESID ? kFinTt : kFinAp>(part, red, sc, ctl);
 }
 
 // q = A p (vector-CSR, T lanes per row) and p . q
 template <int T, bool PART = false>
 __global__ void __launch_bounds__(kThreads)
 ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const double *__restrict__ v,
-          const double *__restrict__ p, double *__restrict__ q, PcgScalars *sc, Reduce red, PartView pv = PartView()) {
+          const double *__restrict__ p, double *__restrict__ q, PcgScalars *sc, Reduce red, FinCtl ctl,
+          PartView pv = PartView()) {
     pdl_begin();
     block_partials_begin();
     double part[1] = {0.0};
@@ -1009,12 +1006,12 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
             part[0] += p[i] * s;
         }
     }
-    block_partials<1>(part, red);
+    block_partials<1, kFinAp>(part, red, sc, ctl);
 }
 
 __global__ void __launch_bounds__(kThreads)
 xr_update_kernel(int32_t n, const double *__restrict__ p, const double *__restrict__ q, double *__restrict__ x,
-                 double *__restrict__ r, const PcgScalars *sc, Reduce red, CycleInput next, double *__restrict__ xs) {
+                 double *__restrict__ r, PcgScalars *sc, Reduce red, CycleInput next, double *__restrict__ xs, FinCtl ctl) {
     pdl_begin();
     block_partials_begin();
     const double alpha = sc->alpha;
@@ -1040,12 +1037,12 @@ xr_update_kernel(int32_t n, const double *__restrict__ p, const double *__restri
         }
         part[0] += ri * ri;
     }
-    block_partials<1>(part, red);
+    block_partials<1, kFinXr>(part, red, sc, ctl);
 }
 
 __global__ void __launch_bounds__(kThreads)
 rz_kernel(int32_t n, const double *__restrict__ r, const double *__restrict__ z, const double *__restrict__ q,
-          PcgScalars *sc, Reduce red) {
+          PcgScalars *sc, Reduce red, FinCtl ctl) {
     pdl_begin();
     block_partials_begin();
     int first = sc->start;
@@ -1055,14 +1052,14 @@ rz_kernel(int32_t n, const double *__restrict__ r, const double *__restrict__ z,
         part[0] += r[i] * zi;
         if (!first) part[1] += zi * q[i];
     }
-    block_partials<2>(part, red);
+    block_partials<2, kFinRz>(part, red, sc, ctl);
 }
 
 template <int T, bool PART = false>
 __global__ void __launch_bounds__(kThreads)
 resid_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const double *__restrict__ v,
              const double *__restrict__ b, const double *__restrict__ x, double *__restrict__ t_out,
-             PcgScalars *sc, Reduce red, PartView pv = PartView()) {
+             PcgScalars *sc, Reduce red, FinCtl ctl, PartView pv = PartView()) {
     pdl_begin();
     block_partials_begin();
     double part[1] = {0.0};
@@ -1081,7 +1078,7 @@ resid_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restric
             part[0] += e * e;
         }
     }
-    block_partials<1>(part, red);
+    block_partials<1, kFinTt>(part, red, sc, ctl);
 }
 
 // level-0 post-smoothing z = x + d (b - A x) with r.z (r = b) and, for
@@ -1091,7 +1088,7 @@ template <int T, bool ZQ, bool PART = false>
 __global__ void __launch_bounds__(kThreads)
 post_rz_csr_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const double *__restrict__ v,
                    const double *__restrict__ x, const double *__restrict__ b, const double *__restrict__ dinv,
-                   double *__restrict__ z, const double *__restrict__ q, PcgScalars *sc, Reduce red,
+                   double *__restrict__ z, const double *__restrict__ q, PcgScalars *sc, Reduce red, FinCtl ctl,
                    PartView pv = PartView()) {
     pdl_begin();
     block_partials_begin();
@@ -1116,7 +1113,7 @@ post_rz_csr_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__r
             if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
         }
     }
-    block_partials<ZQ ? 2 : 1>(part, red);
+    block_partials<ZQ ? 2 : 1, kFinRz>(part, red, sc, ctl);
 }
 
 template <bool D16, bool ZQ>
@@ -1124,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads)
 post_rz_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ soff,
                     const int32_t *__restrict__ sw, SellIdx ix, const double *__restrict__ sv,
                     const double *__restrict__ x, const double *__restrict__ b, const double *__restrict__ dinv,
-                    double *__restrict__ z, const double *__restrict__ q, PcgScalars *sc, Reduce red) {
+                    double *__restrict__ z, const double *__restrict__ q, PcgScalars *sc, Reduce red, FinCtl ctl) {
     pdl_begin();
     block_partials_begin();
     double part[ZQ ? 2 : 1];
@@ -1143,13 +1140,13 @@ post_rz_sell_kernel(int32_t n, const int32_t *__restrict__ perm, const int32_t *
         part[0] += bi * zi;
         if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
     }
-    block_partials<ZQ ? 2 : 1>(part, red);
+    block_partials<ZQ ? 2 : 1, kFinRz>(part, red, sc, ctl);
 }
 
 template <bool ZQ>
 __global__ void __launch_bounds__(kThreads, kPatBlocks)
 post_rz_pat_kernel(int32_t n, PatView<double> pt, const double *x, const double *b, double *z, const double *q,
-                   PcgScalars *sc, Reduce red) {
+                   PcgScalars *sc, Reduce red, FinCtl ctl) {
     block_partials_begin();
     const PatSmem<double> t = pat_begin(pt);
     double part[ZQ ? 2 : 1];
@@ -1164,7 +1161,7 @@ post_rz_pat_kernel(int32_t n, PatView<double> pt, const double *x, const double 
         part[0] += bi * zi;
         if (ZQ) part[ZQ ? 1 : 0] += zi * q[i];
     });
-    block_partials<ZQ ? 2 : 1>(part, red);
+    block_partials<ZQ ? 2 : 1, kFinRz>(part, red, sc, ctl);
 }
 
 // r.z and z.q of the FP32 cycle's output, which stays in FP32 (the search
@@ -1172,7 +1169,7 @@ post_rz_pat_kernel(int32_t n, PatView<double> pt, const double *x, const double 
 // and read)
 __global__ void __launch_bounds__(kThreads)
 rz32_kernel(int32_t n, const float *__restrict__ z32, const double *__restrict__ r, const double *__restrict__ q,
-            PcgScalars *sc, Reduce red) {
+            PcgScalars *sc, Reduce red, FinCtl ctl) {
     pdl_begin();
     block_partials_begin();
     double part[2] = {0.0, 0.0};
@@ -1181,7 +1178,7 @@ rz32_kernel(int32_t n, const float *__restrict__ z32, const double *__restrict__
         part[0] += r[i] * zi;
         part[1] += zi * q[i];
     }
-    block_partials<2>(part, red);
+    block_partials<2, kFinRz>(part, red, sc, ctl);
 }
 
 template <typename XT>
@@ -1394,8 +1391,8 @@ template void pcg_p_update<float>(int32_t, const float *, double *, const PcgSca
 template <int T>
 static void launch_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc, Reduce red, cudaStream_t s) {
     int blocks = reduce_blocks((int64_t)A.nrows * T);
-    { pdl_launch(ap_kernel<T>, blocks, kThreads, 0, s, A.nrows, A.rp, A.ci, A.v, p, q, sc, red, PartView()); ::amg::count_launch(); }
-    launch_finish<1, kFinAp>(blocks, red, sc, s);
+    { pdl_launch(ap_kernel<T>, blocks, kThreads, 0, s, A.nrows, A.rp, A.ci, A.v, p, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); }
+    launch_finish<1, kFinAp>(blocks, red, sc, s, fin_ctl(blocks));
 }
 
 // the SELL forms of A p and of the true residual; returns the block count
@@ -1403,16 +1400,17 @@ template <bool RESID>
 static int launch_ap_sell(const CycMat<double> &A, const double *p, const double *b, double *q, PcgScalars *sc,
                           Reduce red, cudaStream_t s) {
     const int blocks = reduce_blocks(A.nrows);
+    const FinCtl ctl = fin_ctl(blocks);
     const SellIdx ix{A.sci, A.sd};
     const bool sh = A.max_row > 0 && A.max_row <= kShortMax;
     if (A.sd && sh)
-        { pdl_launch(ap_sell_kernel<true, true, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red); ::amg::count_launch(); }
+        { pdl_launch(ap_sell_kernel<true, true, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red, ctl); ::amg::count_launch(); }
     else if (A.sd)
-        { pdl_launch(ap_sell_kernel<true, false, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red); ::amg::count_launch(); }
+        { pdl_launch(ap_sell_kernel<true, false, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red, ctl); ::amg::count_launch(); }
     else if (sh)
-        { pdl_launch(ap_sell_kernel<false, true, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red); ::amg::count_launch(); }
+        { pdl_launch(ap_sell_kernel<false, true, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red, ctl); ::amg::count_launch(); }
     else
-        { pdl_launch(ap_sell_kernel<false, false, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red); ::amg::count_launch(); }
+        { pdl_launch(ap_sell_kernel<false, false, RESID>, blocks, kThreads, 0, s, A.nrows, A.perm, A.soff, A.sw, ix, A.sv, p, b, q, sc, red, ctl); ::amg::count_launch(); }
     return blocks;
 }
 
@@ -1420,21 +1418,21 @@ void pcg_ap(const CycMat<double> &A, const double *p, double *q, PcgScalars *sc,
     if (A.part.parts) {  // row-partitioned: exchange, then the one-lane kernel's loop
         part_exchange(A.part, p, s);
         const int blocks = reduce_blocks(A.nrows);
-        { pdl_launch(ap_kernel<1, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, p, q, sc, red, A.part); ::amg::count_launch(); }
-        launch_finish<1, kFinAp>(blocks, red, sc, s);
+        { pdl_launch(ap_kernel<1, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, p, q, sc, red, fin_ctl(blocks), A.part); ::amg::count_launch(); }
+        launch_finish<1, kFinAp>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     if (A.pat.pid) {
         const int blocks = pat_grid(A.nrows);
-        { pdl_launch(ap_pat_kernel<false>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, p, (const double *)nullptr, q, sc, red); ::amg::count_launch(); }
-        launch_finish<1, kFinAp>(blocks, red, sc, s);
+        { pdl_launch(ap_pat_kernel<false>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, p, (const double *)nullptr, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+        launch_finish<1, kFinAp>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     if (A.variant == AMG_SPMV_SELL32 && A.sv && A.sell_c == 32) {
         const int blocks = launch_ap_sell<false>(A, p, nullptr, q, sc, red, s);
-        launch_finish<1, kFinAp>(blocks, red, sc, s);
+        launch_finish<1, kFinAp>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
@@ -1453,8 +1451,9 @@ void pcg_xr_update(int32_t n, const double *p, const double *q, double *x, doubl
                    Reduce red, cudaGraphConditionalHandle handle, bool use_handle, const CycleInput &next,
                    double *xs, cudaStream_t s) {
     int blocks = reduce_blocks(n);
-    { pdl_launch(xr_update_kernel, blocks, kThreads, 0, s, n, p, q, x, r, sc, red, next, xs); ::amg::count_launch(); }
-    launch_finish<1, kFinXr>(blocks, red, sc, s, handle, use_handle);
+    const FinCtl ctl = fin_ctl(blocks, handle, use_handle);
+    { pdl_launch(xr_update_kernel, blocks, kThreads, 0, s, n, p, q, x, r, sc, red, next, xs, ctl); ::amg::count_launch(); }
+    launch_finish<1, kFinXr>(blocks, red, sc, s, ctl);
     AMG_CHECK_LAUNCH();
 }
 
@@ -1466,15 +1465,15 @@ static void post_smooth_rz_launch(const CycMat<double> &A, const double *x, cons
     if (A.part.parts) {
         part_exchange(A.part, x, s);
         const int blocks = reduce_blocks(n);
-        { pdl_launch(post_rz_csr_kernel<1, ZQ, true>, blocks, kThreads, 0, s, n, A.rp, A.part.cext, A.v, x, b, dinv, z, q, sc, red, A.part); ::amg::count_launch(); }
-        launch_finish<NV, kFinRz>(blocks, red, sc, s);
+        { pdl_launch(post_rz_csr_kernel<1, ZQ, true>, blocks, kThreads, 0, s, n, A.rp, A.part.cext, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), A.part); ::amg::count_launch(); }
+        launch_finish<NV, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     if (A.pat.pid) {
         const int blocks = pat_grid(n);
-        { pdl_launch(post_rz_pat_kernel<ZQ>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, n, A.pat, x, b, z, q, sc, red); ::amg::count_launch(); }
-        launch_finish<NV, kFinRz>(blocks, red, sc, s);
+        { pdl_launch(post_rz_pat_kernel<ZQ>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, n, A.pat, x, b, z, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+        launch_finish<NV, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
@@ -1482,24 +1481,24 @@ static void post_smooth_rz_launch(const CycMat<double> &A, const double *x, cons
         int blocks = reduce_blocks(n);
         const SellIdx ix{A.sci, A.sd};
         if (A.sd)
-            { pdl_launch(post_rz_sell_kernel<true, ZQ>, blocks, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, x, b, dinv, z, q, sc, red); ::amg::count_launch(); }
+            { pdl_launch(post_rz_sell_kernel<true, ZQ>, blocks, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, x, b, dinv, z, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
         else
-            { pdl_launch(post_rz_sell_kernel<false, ZQ>, blocks, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, x, b, dinv, z, q, sc, red); ::amg::count_launch(); }
-        launch_finish<NV, kFinRz>(blocks, red, sc, s);
+            { pdl_launch(post_rz_sell_kernel<false, ZQ>, blocks, kThreads, 0, s, n, A.perm, A.soff, A.sw, ix, A.sv, x, b, dinv, z, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+        launch_finish<NV, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     int T = threads_per_row(A.variant);
     int blocks = reduce_blocks((int64_t)n * T);
     switch (T) {
-        case 1: { pdl_launch(post_rz_csr_kernel<1, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
-        case 2: { pdl_launch(post_rz_csr_kernel<2, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
-        case 4: { pdl_launch(post_rz_csr_kernel<4, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
-        case 8: { pdl_launch(post_rz_csr_kernel<8, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
-        case 16: { pdl_launch(post_rz_csr_kernel<16, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
-        default: { pdl_launch(post_rz_csr_kernel<32, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, PartView()); ::amg::count_launch(); } break;
+        case 1: { pdl_launch(post_rz_csr_kernel<1, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
+        case 2: { pdl_launch(post_rz_csr_kernel<2, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
+        case 4: { pdl_launch(post_rz_csr_kernel<4, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
+        case 8: { pdl_launch(post_rz_csr_kernel<8, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
+        case 16: { pdl_launch(post_rz_csr_kernel<16, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
+        default: { pdl_launch(post_rz_csr_kernel<32, ZQ>, blocks, kThreads, 0, s, n, A.rp, A.ci, A.v, x, b, dinv, z, q, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); } break;
     }
-    launch_finish<NV, kFinRz>(blocks, red, sc, s);
+    launch_finish<NV, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
     AMG_CHECK_LAUNCH();
 }
 
@@ -1514,8 +1513,8 @@ bool post_smooth_rz(const CycMat<double> &A, const double *x, const double *b, c
 void pcg_rz32(int32_t n, const float *z32, const double *r, const double *q, PcgScalars *sc, Reduce red,
               cudaStream_t s) {
     int blocks = reduce_blocks(n);
-    { pdl_launch(rz32_kernel, blocks, kThreads, 0, s, n, z32, r, q, sc, red); ::amg::count_launch(); }
-    launch_finish<2, kFinRz>(blocks, red, sc, s);
+    { pdl_launch(rz32_kernel, blocks, kThreads, 0, s, n, z32, r, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+    launch_finish<2, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
     AMG_CHECK_LAUNCH();
 }
 
@@ -1536,8 +1535,8 @@ void to_f32_scaled(int64_t n, const double *src, const float *d, float *dst, flo
 void pcg_rz(int32_t n, const double *r, const double *z, const double *q, PcgScalars *sc, Reduce red,
             cudaStream_t s) {
     int blocks = reduce_blocks(n);
-    { pdl_launch(rz_kernel, blocks, kThreads, 0, s, n, r, z, q, sc, red); ::amg::count_launch(); }
-    launch_finish<2, kFinRz>(blocks, red, sc, s);
+    { pdl_launch(rz_kernel, blocks, kThreads, 0, s, n, r, z, q, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+    launch_finish<2, kFinRz>(blocks, red, sc, s, fin_ctl(blocks));
     AMG_CHECK_LAUNCH();
 }
 
@@ -1546,27 +1545,27 @@ void true_residual(const CycMat<double> &A, const double *b, const double *x, do
     if (A.part.parts) {  // row-partitioned: the four-lane kernel's loop, as below
         part_exchange(A.part, x, s);
         const int blocks = reduce_blocks((int64_t)A.nrows * 4);
-        { pdl_launch(resid_kernel<4, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, b, x, t, sc, red, A.part); ::amg::count_launch(); }
-        launch_finish<1, kFinTt>(blocks, red, sc, s);
+        { pdl_launch(resid_kernel<4, true>, blocks, kThreads, 0, s, A.nrows, A.rp, A.part.cext, A.v, b, x, t, sc, red, fin_ctl(blocks), A.part); ::amg::count_launch(); }
+        launch_finish<1, kFinTt>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     if (A.pat.pid) {
         const int blocks = pat_grid(A.nrows);
-        { pdl_launch(ap_pat_kernel<true>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, x, b, t, sc, red); ::amg::count_launch(); }
-        launch_finish<1, kFinTt>(blocks, red, sc, s);
+        { pdl_launch(ap_pat_kernel<true>, blocks, kThreads, pat_smem_bytes<double>(A.pat.npat, A.pat.width), s, A.nrows, A.pat, x, b, t, sc, red, fin_ctl(blocks)); ::amg::count_launch(); }
+        launch_finish<1, kFinTt>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     if (A.variant == AMG_SPMV_SELL32 && A.sv && A.sell_c == 32) {  // the operator's tuned SELL copy, as A p uses
         const int blocks = launch_ap_sell<true>(A, x, b, t, sc, red, s);
-        launch_finish<1, kFinTt>(blocks, red, sc, s);
+        launch_finish<1, kFinTt>(blocks, red, sc, s, fin_ctl(blocks));
         AMG_CHECK_LAUNCH();
         return;
     }
     int blocks = reduce_blocks((int64_t)A.nrows * 4);
-    { pdl_launch(resid_kernel<4>, blocks, kThreads, 0, s, A.nrows, A.rp, A.ci, A.v, b, x, t, sc, red, PartView()); ::amg::count_launch(); }
-    launch_finish<1, kFinTt>(blocks, red, sc, s);
+    { pdl_launch(resid_kernel<4>, blocks, kThreads, 0, s, A.nrows, A.rp, A.ci, A.v, b, x, t, sc, red, fin_ctl(blocks), PartView()); ::amg::count_launch(); }
+    launch_finish<1, kFinTt>(blocks, red, sc, s, fin_ctl(blocks));
     AMG_CHECK_LAUNCH();
 }
 

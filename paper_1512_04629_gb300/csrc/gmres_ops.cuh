@@ -20,6 +20,7 @@ struct GmresScalars {
     double thresh;  // tol ||b||: stop when the residual estimate reaches it
     double est;     // |g_j|, the residual norm of the cycle's current iterate
     double hn;      // ||w|| of the last step (h_{j+1,j})
+    double rhn;     // 1 / hn
     double tt;      // ||b - A x||^2 of the last true residual
     double ww;      // ||w||^2 before orthogonalisation
     double wn2;     // ||w||^2 after the first pass
@@ -58,12 +59,16 @@ void mdot(int64_t n, int m, const double *V, const double *w, GmresScalars *sc, 
 // j += 1, and the WHILE condition when `use_handle`.
 void mupdate(int64_t n, int m, const double *V, double *w, GmresScalars *sc, GmresArrays ar, bool second,
              cudaGraphConditionalHandle handle, bool use_handle, cudaStream_t s);
-// v_j = w / hn into V (row j) and into `next` (the next cycle input)
-void normalize(int64_t n, const double *w, double *V, double *next, const GmresScalars *sc, cudaStream_t s);
+// v_j = w / hn into V (row j) and into `next` (the next cycle input); with x0
+// also its level-0 pre-smooth x0 = dinv0 .* v_j
+void normalize(int64_t n, const double *w, double *V, double *next, const GmresScalars *sc, const double *dinv0,
+               double *x0, cudaStream_t s);
 // Z row j = z (before the step finisher increments j)
 void store_z(int64_t n, const double *z, double *Z, const GmresScalars *sc, cudaStream_t s);
 // new cycle: v_0 = r / beta into V and next, g = beta e_1, j = 0 (beta from sc->tt)
-void start(int64_t n, const double *r, double *V, double *next, GmresScalars *sc, GmresArrays ar, cudaStream_t s);
+// (x0 as for normalize)
+void start(int64_t n, const double *r, double *V, double *next, GmresScalars *sc, GmresArrays ar, const double *dinv0,
+           double *x0, cudaStream_t s);
 // x = x0 + Z y with R y = g over the cycle's j columns
 void form_x(int64_t n, int m, const double *Z, const double *x0, double *x, GmresScalars *sc, GmresArrays ar,
             cudaStream_t s);

@@ -1439,6 +1439,11 @@ struct GmRun {
 GmresArrays gm_arrays(Hierarchy &h) { return gmres_arrays(h.garr.as<double>(), h.gm_m); }
 GmresScalars *gm_dsc(Hierarchy &h) { return h.gsc.as<GmresScalars>(); }
 
+// where an FP64 cycle keeps its level-0 pre-smooth (null: none, or FP32)
+double *gm_x0(Hierarchy &h) {
+    return h.opt.precision == AMG_PREC_FP64 && h.nlev() > 1 ? h.lev[0]->x.as<double>() : nullptr;
+}
+
 void gm_read(Hierarchy &h, cudaStream_t s) {
     AMG_CUDA(cudaMemcpyAsync(h.h_gsc, gm_dsc(h), sizeof(GmresScalars), cudaMemcpyDeviceToHost, s));
     AMG_CUDA(cudaStreamSynchronize(s));
@@ -1471,7 +1476,9 @@ void gm_step(Hierarchy &h, cudaStream_t s, cudaGraphConditionalHandle handle, bo
     GmresArrays ar = gm_arrays(h);
     GmresScalars *sc = gm_dsc(h);
     double *V = h.gV.as<double>(), *Z = h.gZ.as<double>(), *w = h.pq.as<double>();
-    vcycle_f64(h, h.pr.as<double>(), h.pz.as<double>(), s);
+    CycleCtl ctl;
+    ctl.x0_ready = gm_x0(h) != nullptr;  // written with the basis vector
+    vcycle_f64(h, h.pr.as<double>(), h.pz.as<double>(), s, ctl);
     timed(h, 6, 0, 16.0 * n, s, [&] { gm::store_z(n, h.pz.as<double>(), Z, sc, s); });
     CycMat<double> A0 = a0_mat(h);
     const double ap_bytes = (double)A0.nnz * 12 + 4.0 * (n + 1) + 16.0 * n;
@@ -1481,7 +1488,7 @@ void gm_step(Hierarchy &h, cudaStream_t s, cudaGraphConditionalHandle handle, bo
         gm::mupdate(n, m, V, w, sc, ar, false, handle, false, s);
         gm::mdot(n, m, V, w, sc, ar, true, s);
         gm::mupdate(n, m, V, w, sc, ar, true, handle, use_handle, s);
-        gm::normalize(n, w, V, h.pr.as<double>(), sc, s);
+        gm::normalize(n, w, V, h.pr.as<double>(), sc, h.lev[0]->dinv.as<double>(), gm_x0(h), s);
     });
 }
 
@@ -1539,7 +1546,8 @@ double gm_start(Hierarchy &h, const double *b, double thresh, cudaStream_t s, do
     c.thresh = thresh;
     c.tt = rn * rn;
     gm_write(h, s);
-    gm::start(n, h.pt.as<double>(), h.gV.as<double>(), h.pr.as<double>(), gm_dsc(h), gm_arrays(h), s);
+    gm::start(n, h.pt.as<double>(), h.gV.as<double>(), h.pr.as<double>(), gm_dsc(h), gm_arrays(h),
+              h.lev[0]->dinv.as<double>(), gm_x0(h), s);
     gm_read(h, s);
     return rn;
 }
