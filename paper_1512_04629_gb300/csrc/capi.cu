@@ -242,10 +242,7 @@ amg_status amg_sparsify(amg_hierarchy *H, const double *gamma, int n_gamma) {
         require(h.opt.method != AMG_METHOD_NONGALERKIN, "a non-Galerkin hierarchy retains no Galerkin operator");
         cudaStream_t s = nullptr;
         AllocOn alloc_scope(s);
-        apply_gammas(h, gamma, n_gamma, s);
-        std::vector<int> all;
-        for (int l = 0; l < h.nlev(); ++l) all.push_back(l);
-        prepare_cycle(h, s, all);
+        sparsify_again(h, gamma, n_gamma, s);
         return AMG_OK;
     });
 }

@@ -276,8 +276,11 @@ static const uint8_t *hybrid_pattern(Hierarchy &h, int l, cudaStream_t s) {
     return V.inM_hybrid.as<uint8_t>();
 }
 
-static void resparsify_one(Hierarchy &h, Level &V, int l, cudaStream_t s) {
+// park: receives the operator that is replaced (its buffers' releases wait for
+// the device one by one; the caller returns them together)
+static void resparsify_one(Hierarchy &h, Level &V, int l, cudaStream_t s, std::vector<DevCSR> *park = nullptr) {
     if (l == 0 || V.gamma == 0.0) {
+        if (park) park->push_back(std::move(V.H));
         V.H = DevCSR();
         V.h_alias = true;
         AMG_CUDA(cudaMemsetAsync(V.keep.ptr, 1, V.A.nnz, s));
@@ -293,17 +296,18 @@ static void resparsify_one(Hierarchy &h, Level &V, int l, cudaStream_t s) {
     }
     setup::sparsify(V.A, inM, V.tpos.as<int32_t>(), V.diagpos.as<int32_t>(), V.gamma, V.keep.as<uint8_t>(), H, s,
                     S.as<uint8_t>());
+    if (park) park->push_back(std::move(V.H));
     V.H = std::move(H);
     V.h_alias = false;
 }
-
-void resparsify_level(Hierarchy &h, int l, cudaStream_t s) { resparsify_one(h, *h.lev[l], l, s); }
 
 static double level_gamma(const double *gamma, int n_gamma, int l) {
     return (l > 0 && n_gamma > 0 && gamma) ? gamma[std::min(l, n_gamma - 1)] : 0.0;
 }
 
-void apply_gammas(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s) {
+static void drop_relaxed(Hierarchy &h, std::vector<DevCSR> &old, const std::vector<int> &levels);
+
+void apply_gammas(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s, std::vector<DevCSR> *park) {
     if (h.opt.method == AMG_METHOD_NONGALERKIN) {  // thinned during the setup: every level is final
         for (int l = 0; l < h.nlev(); ++l) {
             Level &V = *h.lev[l];
@@ -315,8 +319,19 @@ void apply_gammas(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s
     }
     for (int l = 0; l < h.nlev(); ++l) {
         h.lev[l]->gamma = level_gamma(gamma, n_gamma, l);
-        timed(h, 13, l, 0.0, s, [&] { resparsify_level(h, l, s); });
+        timed(h, 13, l, 0.0, s, [&] { resparsify_one(h, *h.lev[l], l, s, park); });
     }
+}
+
+// amg_sparsify: every level again, and the cycle data of those whose operator
+// may have changed -- all but the finest, which is never sparsified
+void sparsify_again(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s) {
+    std::vector<DevCSR> old;
+    apply_gammas(h, gamma, n_gamma, s, &old);
+    std::vector<int> levels;
+    for (int l = 1; l < h.nlev(); ++l) levels.push_back(l);
+    drop_relaxed(h, old, levels);
+    prepare_cycle(h, s, levels);
 }
 
 // Algorithm 5 drop-tolerance update (finest level >= 1 with gamma > 0, s
@@ -328,13 +343,15 @@ int reintroduce(Hierarchy &h, int s_levels, cudaStream_t s) {
     for (int l = 1; l < L; ++l)
         if (h.lev[l]->gamma > 0.0) { lstart = l; break; }
     if (lstart < 0) return 0;
+    std::vector<DevCSR> old;
     std::vector<int> changed;
     for (int l = lstart; l < lstart + s_levels && l < L; ++l) {
         double g = h.lev[l]->gamma / 10.0;
         h.lev[l]->gamma = (g >= h.opt.gamma_min * (1.0 - 1e-12)) ? g : 0.0;
-        timed(h, 13, l, 0.0, s, [&] { resparsify_level(h, l, s); });
+        timed(h, 13, l, 0.0, s, [&] { resparsify_one(h, *h.lev[l], l, s, &old); });
         changed.push_back(l);
     }
+    drop_relaxed(h, old, changed);
     prepare_cycle(h, s, changed);
     return (int)changed.size();
 }
@@ -409,6 +426,27 @@ static void free_sell(Level &V) {
     V.pid.release(); V.ptab.release();
     V.npat = V.pwidth = 0;
     V.sell_entries = 0;
+}
+
+// the cycle's copies of a level's relaxed operator
+static void drop_operator_copies(Level &V) {
+    V.hv32.release();
+    V.hv16.release();
+    free_sell(V);
+}
+
+// After levels were sparsified again: their former operators and the cycle's
+// copies of them go back to the pool after one wait for the device --
+// released one by one, each buffer waits for it (a dozen per level).
+static void drop_relaxed(Hierarchy &h, std::vector<DevCSR> &old, const std::vector<int> &levels) {
+    int cur = -1;
+    cudaGetDevice(&cur);
+    if (cur != h.device) return;  // the releases wait for themselves
+    AMG_CUDA(cudaDeviceSynchronize());
+    IdleRelease idle;
+    idle.enter();
+    old.clear();
+    for (int l : levels) drop_operator_copies(*h.lev[l]);
 }
 
 // Autotuner: time the post-smoothing kernel of one level under each plausible
@@ -524,8 +562,14 @@ template <typename VT, typename XT> static void autotune_level(Hierarchy &h, Lev
     (void)h;
 }
 
+// a buffer of exactly these bytes: the one there is, when it is (a level that
+// is prepared again keeps its vectors; its contents are written anew)
+static void ensure_bytes(DevBuf &b, size_t bytes) {
+    if (!b.ptr || b.bytes != bytes) b.alloc(bytes);
+}
+
 template <typename T> static void alloc_zero(DevBuf &b, int64_t n, cudaStream_t s) {
-    b.alloc(sizeof(T) * (size_t)(n + kPad));
+    ensure_bytes(b, sizeof(T) * (size_t)(n + kPad));
     AMG_CUDA(cudaMemsetAsync(b.ptr, 0, b.bytes, s));
 }
 
@@ -536,21 +580,18 @@ static bool prepare_level_at(Hierarchy &h, Level &V, int l, bool has_p, cudaStre
     const DevCSR &M = V.op();
     int32_t n = V.n();
     int prec = h.opt.precision;
-    V.l1.alloc(sizeof(double) * (n + kPad));
-    V.dinv.alloc(sizeof(double) * (n + kPad));
+    ensure_bytes(V.l1, sizeof(double) * (n + kPad));
+    ensure_bytes(V.dinv, sizeof(double) * (n + kPad));
     setup::l1_diag(M, V.l1.as<double>(), V.dinv.as<double>(), s);
     V.vbytes = prec == AMG_PREC_FP64 ? 8 : (prec == AMG_PREC_FP32_BF16 && l >= 2 ? 2 : 4);
-    V.hv32.release();
-    V.hv16.release();
-    V.dinv32.release();
-    free_sell(V);
+    drop_operator_copies(V);
     if (prec == AMG_PREC_FP64) {
         alloc_zero<double>(V.b, n, s); alloc_zero<double>(V.x, n, s);
         alloc_zero<double>(V.r, n, s); alloc_zero<double>(V.xo, n, s);
     } else {
         alloc_zero<float>(V.b, n, s); alloc_zero<float>(V.x, n, s);
         alloc_zero<float>(V.r, n, s); alloc_zero<float>(V.xo, n, s);
-        V.dinv32.alloc(sizeof(float) * (n + kPad));
+        ensure_bytes(V.dinv32, sizeof(float) * (n + kPad));
         cyc::convert_values<float>(V.dinv.as<double>(), V.dinv32.as<float>(), n, s);
         if (V.vbytes == 4) {
             V.hv32.alloc(sizeof(float) * (M.nnz + kPad));
@@ -1359,6 +1400,13 @@ void ensure_graph(Hierarchy &h) {
     h.graph_dirty = false;
 }
 
+// A run of at most this many steps (a window of Algorithm 5) on a hierarchy
+// that has changed since its graph was built is launched kernel by kernel:
+// nearly every window ends in a reintroduction, and capturing and
+// instantiating the step costs what several eager steps do (adaptive solves
+// from gamma = 1, windows of 3: 75^3 9.5 -> 8.4 ms, 128^3 21.3 -> 19.9 ms).
+constexpr int kEagerSteps = 4;
+
 // Runs up to max_steps CG steps (stopping at the recurrence test, then
 // confirming with the true residual; a failed confirmation replaces r).
 // divf > 0 adds the divergence test (Section 6: with too many entries
@@ -1371,7 +1419,7 @@ void pcg_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int ma
     run = Run();
     run.rnorm = rnorm_now;
     if (rnorm_now <= tol * bnorm) { run.converged = true; return; }
-    bool graph = h.opt.use_graph && !h.timing;
+    bool graph = h.opt.use_graph && !h.timing && !(max_steps <= kEagerSteps && h.graph_dirty);
     if (graph) ensure_graph(h);
     double thresh2 = (tol * bnorm) * (tol * bnorm);
     int32_t n = h.lev[0]->n();
@@ -1569,7 +1617,7 @@ void gm_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int max
     GmresScalars &c = *h.h_gsc;
     run.rnorm = c.est;
     if (c.est <= thresh) { run.converged = true; return; }
-    const bool graph = h.opt.use_graph && !h.timing;
+    const bool graph = h.opt.use_graph && !h.timing && !(max_steps <= kEagerSteps && h.g_gmres_version != h.version);
     if (graph) gm_ensure_graph(h);
     while (run.steps < max_steps) {
         if (c.j == h.gm_m) {  // restart

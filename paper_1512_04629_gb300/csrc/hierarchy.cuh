@@ -294,8 +294,9 @@ void setup_hierarchy(Hierarchy &h, cudaStream_t s, const double *gamma, int n_ga
 void assemble_levels(Hierarchy &h, std::vector<DevCSR> &A, std::vector<DevCSR> &P,
                      const std::vector<std::vector<int8_t>> &cf,
                      const std::vector<std::vector<uint8_t>> &inM, cudaStream_t s);
-void apply_gammas(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s);
-void resparsify_level(Hierarchy &h, int l, cudaStream_t s);
+void apply_gammas(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s,
+                  std::vector<DevCSR> *park = nullptr);
+void sparsify_again(Hierarchy &h, const double *gamma, int n_gamma, cudaStream_t s);
 void prepare_cycle(Hierarchy &h, cudaStream_t s, const std::vector<int> &levels);
 void ensure_workspace(Hierarchy &h, cudaStream_t s);
 int reintroduce(Hierarchy &h, int s_levels, cudaStream_t s);
