@@ -195,6 +195,17 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t key) {
 
 enum : int8_t { kU = 0, kC = 1, kF = -1 };
 
+// The spare entries after a CSR array's nnz, zeroed by the kernel that fills
+// the array instead of two memsets an array pair: at the small levels a
+// setup's time is its launches and host round trips.
+__device__ __forceinline__ void zero_pad(int64_t nnz, int32_t *ci, double *v) {
+    static_assert(kPad <= 32, "one warp of any block");
+    if (blockIdx.x == 0 && threadIdx.x < kPad) {
+        ci[nnz + threadIdx.x] = 0;
+        v[nnz + threadIdx.x] = 0.0;
+    }
+}
+
 // Appends row i to a list when `keep` holds, with one global atomic per
 // block (warps reserve their places in shared memory first): a global
 // counter that every warp of a large grid increments serialises on one
@@ -214,6 +225,11 @@ __device__ __forceinline__ void block_append(bool keep, int32_t i, int32_t *list
     if (threadIdx.x == 0) s_base = s_count ? atomicAdd(count, s_count) : 0;
     __syncthreads();
     if (keep) list[s_base + wbase + __popc(m & ((1u << lane) - 1u))] = i;
+}
+
+__device__ __forceinline__ double pmis_weight(int32_t cnt, uint64_t seed, int32_t level, int32_t i) {
+    const uint64_t key = seed ^ ((uint64_t)(uint32_t)level << 40) ^ (uint64_t)i;
+    return (double)cnt + (double)(splitmix64(key) >> 11) * (1.0 / 9007199254740992.0);
 }
 
 template <int T>
@@ -249,9 +265,7 @@ __global__ void pmis_init_kernel(int32_t n, const int32_t *rp, const int32_t *tp
     cnt = group_sum_i32<T>(cnt);
     bool und = false;
     if (live && t == 0) {
-        uint64_t key = seed ^ ((uint64_t)(uint32_t)level << 40) ^ (uint64_t)i;
-        double u = (double)(splitmix64(key) >> 11) * (1.0 / 9007199254740992.0);
-        w[i] = (double)cnt + u;
+        w[i] = pmis_weight(cnt, seed, level, i);
         state[i] = cnt == 0 ? kF : kU;
         und = cnt != 0;
     }
@@ -367,6 +381,122 @@ __global__ void pmis_apply_kernel(const int32_t *list, const int *len, int32_t n
     }
 }
 
+// The whole split of a small level in one block: weights, states and the
+// round's selection in shared memory, the rounds separated by block barriers,
+// and the coarse numbering scanned at the end.  out[0] = C points, out[1] =
+// rows left undecided (0, unless a round decided nothing).  The rounds are
+// those of the kernels above -- every row still undecided takes part -- so
+// the split is the same.  A small level's split is launches: one here instead
+// of twenty (a clear, the weights, eight rounds of two, the C flags, their
+// scan).  One block pays about half a microsecond for every 128 rows of a
+// sweep, so the line lies where both cost the same.  Whole setups, the split
+// in launches -> in one block (median ms): 32 x 32 1.62 -> 1.47, 45 x 45
+// 1.77 -> 1.62, 101 x 101 2.26 -> 2.10, 128^3 9.68 -> 9.61.  With the line at
+// 1024 rows the 45 x 45 one takes 1.69; at 4096 the 101 x 101 one 2.20 and the
+// 128^3 one 10.0.
+constexpr int kPmisSmall = 2048, kPmisThreads = 1024;
+template <int T>
+__global__ void __launch_bounds__(kPmisThreads)
+pmis_small_kernel(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *tpos, const uint8_t *strong,
+                  uint64_t seed, int32_t level, uint8_t *sym, int8_t *cf, int32_t *cmap, int *out) {
+    constexpr int kRows = kPmisThreads / T;  // rows of one sweep
+    __shared__ int64_t w[kPmisSmall];        // weights >= 0 order like their bits
+    __shared__ int8_t state[kPmisSmall];
+    __shared__ uint8_t newc[kPmisSmall];
+    __shared__ int s_und[2], s_warp[kPmisThreads / 32];
+    const int t = threadIdx.x % T, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x < 2) s_und[threadIdx.x] = 0;
+    __syncthreads();
+    for (int32_t base = 0; base < n; base += kRows) {  // every lane takes every sweep: group reductions
+        const int32_t i = base + (int32_t)threadIdx.x / T;
+        const bool live = i < n;
+        const int32_t p0 = live ? rp[i] : 0, p1 = live ? rp[i + 1] : 0;
+        int32_t cnt = 0;  // |S^T_i|
+        for (int32_t p = p0 + t; p < p1; p += T) {
+            const uint8_t st = strong[tpos[p]];
+            cnt += st;
+            sym[p] = (uint8_t)(st | strong[p]);  // j in S_i u S^T_i
+        }
+        cnt = group_sum_i32<T>(cnt);
+        if (live && t == 0) {
+            w[i] = __double_as_longlong(pmis_weight(cnt, seed, level, i));
+            state[i] = cnt == 0 ? kF : kU;
+            if (cnt != 0) atomicAdd(&s_und[0], 1);
+        }
+    }
+    __syncthreads();
+    int und = s_und[0], left = und;
+    for (int r = 1; und > 0; ++r) {
+        for (int32_t base = 0; base < n; base += kRows) {
+            const int32_t i = base + (int32_t)threadIdx.x / T;
+            const bool live = i < n && state[i] == kU;
+            bool lose = false;
+            if (live) {
+                const int32_t p1 = rp[i + 1];
+                const int64_t wi = w[i];
+                for (int32_t p = rp[i] + t; p < p1; p += T) {
+                    const int32_t j = ci[p];
+                    const int64_t wj = w[j];
+                    if (sym[p] && state[j] == kU && (wj > wi || (wj == wi && j > i))) lose = true;
+                }
+            }
+            lose = group_any<T>(lose);
+            if (live && t == 0) newc[i] = (uint8_t)!lose;
+        }
+        if (threadIdx.x == 0) s_und[r & 1] = 0;
+        __syncthreads();
+        for (int32_t base = 0; base < n; base += kRows) {
+            const int32_t i = base + (int32_t)threadIdx.x / T;
+            const bool live = i < n && state[i] == kU;  // written by this row's own group only
+            const bool c = live && newc[i];
+            bool f = false;
+            if (live && !c) {
+                const int32_t p1 = rp[i + 1];
+                for (int32_t p = rp[i] + t; p < p1; p += T) {
+                    const int32_t j = ci[p];
+                    const int8_t sj = *(volatile const int8_t *)&state[j];
+                    if (strong[p] && (sj == kC || (sj == kU && newc[j]))) f = true;
+                }
+            }
+            f = group_any<T>(f);
+            if (live && t == 0) {
+                if (c) state[i] = kC;
+                else if (f) state[i] = kF;
+                else atomicAdd(&s_und[r & 1], 1);
+            }
+        }
+        __syncthreads();
+        left = s_und[r & 1];
+        if (left >= und) break;  // no progress: reported, never looped on
+        und = left;
+    }
+    // cmap: the exclusive scan of the C flags, its total last
+    int total = 0;
+    for (int32_t base = 0; base < n; base += kPmisThreads) {
+        const int32_t i = base + (int32_t)threadIdx.x;
+        const bool c = i < n && state[i] == kC;
+        const unsigned m = __ballot_sync(0xffffffffu, c);
+        if (lane == 0) s_warp[wid] = __popc(m);
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int k = 0; k < kPmisThreads / 32; ++k) {
+            if (k < wid) before += s_warp[k];
+            all += s_warp[k];
+        }
+        if (i < n) {
+            cf[i] = state[i];
+            cmap[i] = total + before + __popc(m & ((1u << lane) - 1u));
+        }
+        total += all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        cmap[n] = total;
+        out[0] = total;
+        out[1] = left;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // coarse numbering
 // ---------------------------------------------------------------------------
@@ -409,7 +539,8 @@ __global__ void interp_count_kernel(int32_t n, const int32_t *rp, const int32_t 
 __global__ void interp_rows_kernel(int32_t n, const int32_t *rp, const int32_t *ci,
                                    const double *v, const uint8_t *strong, const int8_t *cf,
                                    const int32_t *cmap, const int32_t *prp, int32_t *pci,
-                                   double *pv, int32_t *prow, double *coef) {
+                                   double *pv, int32_t *prow, double *coef, int64_t pnnz) {
+    zero_pad(pnnz, pci, pv);
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int32_t pos = prp[i];
@@ -492,7 +623,8 @@ __global__ void col_count_kernel(int64_t nnz, const int32_t *ci, int32_t *cnt) {
 }
 
 __global__ void transpose_fill_kernel(int32_t n, const int32_t *rp, const int32_t *ci,
-                                      const double *v, int32_t *fill, int32_t *tci, double *tv) {
+                                      const double *v, int32_t *fill, int32_t *tci, double *tv, int64_t nnz) {
+    zero_pad(nnz, tci, tv);
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     for (int32_t p = rp[i]; p < rp[i + 1]; ++p) {
@@ -709,18 +841,6 @@ __device__ int32_t row_numeric(int32_t i, int32_t lane, const int32_t *arp, cons
     return u;
 }
 
-__global__ void spgemm_ub_kernel(int32_t n, const int32_t *arp, const int32_t *aci,
-                                 const int32_t *bbeg, const int32_t *bend, int64_t *ub) {
-    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t s = 0;
-    for (int32_t p = arp[i]; p < arp[i + 1]; ++p) {
-        int32_t k = aci[p];
-        s += bend[k] - bbeg[k];
-    }
-    ub[i] = s;
-}
-
 constexpr int kBlockHS = 8192, kBlockUmax = 4096, kBlockThreads = 256;
 // Row bins by product bound: three register-sort widths (one row per 8, 16
 // or 32 lanes), two warp hash-accumulator sizes, a block table, a global table.
@@ -741,6 +861,20 @@ struct SpgemmCounts {
     unsigned long long max_ub_global;
     int64_t total_ub;
 };
+
+// Also clears the record that the next kernel counts the bins into.
+__global__ void spgemm_ub_kernel(int32_t n, const int32_t *arp, const int32_t *aci,
+                                 const int32_t *bbeg, const int32_t *bend, int64_t *ub, SpgemmCounts *cnt) {
+    int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *cnt = SpgemmCounts{};
+    if (i >= n) return;
+    int64_t s = 0;
+    for (int32_t p = arp[i]; p < arp[i + 1]; ++p) {
+        int32_t k = aci[p];
+        s += bend[k] - bbeg[k];
+    }
+    ub[i] = s;
+}
 
 __global__ void bin_rows_kernel(int32_t n, const int64_t *ub, int32_t *bins, SpgemmCounts *cnt) {
     __shared__ int32_t local[kNumBins], base[kNumBins];
@@ -1415,7 +1549,8 @@ template <int T>
 __global__ void __launch_bounds__(kThreads)
 sparsify_compact_lanes_kernel(int32_t n, const int32_t *rp, const int32_t *ci, const double *v,
                               const int32_t *diagpos, const uint8_t *keep, const int32_t *hrp, int32_t *hci,
-                              double *hv) {
+                              double *hv, int64_t hnnz) {
+    zero_pad(hnnz, hci, hv);
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t i = (int32_t)(g / T);
     const int t = (int)(g % T);
@@ -1640,7 +1775,9 @@ __global__ void lump_gather_kernel(int32_t n, const int32_t *rp, const int32_t *
 
 // compaction of the kept entries with their gathered values
 __global__ void compact_values_kernel(int32_t n, const int32_t *rp, const int32_t *ci, const uint8_t *keep,
-                                      const double *hval, const int32_t *hrp, int32_t *hci, double *hv) {
+                                      const double *hval, const int32_t *hrp, int32_t *hci, double *hv,
+                                      int64_t hnnz) {
+    zero_pad(hnnz, hci, hv);
     int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int32_t pos = hrp[i];
@@ -1871,7 +2008,8 @@ __global__ void slot_bounds_kernel(int32_t n, const int64_t *obase, const int32_
 }
 
 __global__ void spgemm_compact_kernel(int32_t n, const int64_t *obase, const int32_t *crp, const int32_t *tci,
-                                      const double *tv, int32_t *cci, double *cv) {
+                                      const double *tv, int32_t *cci, double *cv, int64_t nnz) {
+    zero_pad(nnz, cci, cv);
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int32_t i = (int32_t)(g / kCompactLanes);
     int lane = (int)(g % kCompactLanes);
@@ -2000,6 +2138,23 @@ int64_t pmis(const DevCSR &A, const uint8_t *strong, const int32_t *tpos, uint64
         AMG_CUDA(cudaMemsetAsync(cmap, 0, sizeof(int32_t), s));
         return 0;
     }
+    const int T = row_lanes(A, 8);
+    if (n <= kPmisSmall) {
+        TmpBuf sym(A.nnz + 1, s), out(2 * sizeof(int), s);
+        with_row_lanes(T, [&](auto tc) {
+            constexpr int L = decltype(tc)::value;
+            if constexpr (L <= 8) {
+                pmis_small_kernel<L><<<1, kPmisThreads, 0, s>>>(n, A.rp(), A.ci(), tpos, strong, seed, level,
+                                                                sym.as<uint8_t>(), cf, cmap, out.as<int>());
+                ::amg::count_launch();
+            }
+        });
+        AMG_CHECK_LAUNCH();
+        int h[2];
+        read_back(h, out.as<int>(), sizeof(h), s);
+        if (h[1] != 0) throw Error(AMG_ERR_CUDA, "PMIS made no progress");
+        return h[0];
+    }
     // eight rounds per read-back: the levels of the test problems finish
     // within one batch, and a round whose list is empty costs one short launch
     constexpr int kBatch = 8, kMaxRounds = 10000;
@@ -2012,7 +2167,6 @@ int64_t pmis(const DevCSR &A, const uint8_t *strong, const int32_t *tpos, uint64
     int *dc = ccount + 1;
     int32_t *list[2] = {lists.as<int32_t>(), lists.as<int32_t>() + n};
     int g = div_up(n, kThreads);
-    const int T = row_lanes(A, 8);
     const int64_t nres = ::amg::resident_blocks(kThreads);
     AMG_CUDA(cudaMemsetAsync(cnt.ptr, 0, cnt.bytes, s));
     with_row_lanes(T, [&](auto tc) {
@@ -2120,12 +2274,13 @@ void direct_interp(const DevCSR &A, const uint8_t *strong, const int8_t *cf, con
     P.nnz = nnz;
     P.col.alloc(sizeof(int32_t) * (nnz + kPad));
     P.val.alloc(sizeof(double) * (nnz + kPad));
-    AMG_CUDA(cudaMemsetAsync(P.ci() + nnz, 0, sizeof(int32_t) * kPad, s));  // the fill writes rows [0, nnz)
-    AMG_CUDA(cudaMemsetAsync(P.v() + nnz, 0, sizeof(double) * kPad, s));
-    if (n > 0) {
+    if (n == 0) {  // no rows to fill: the spare entries alone
+        AMG_CUDA(cudaMemsetAsync(P.ci() + nnz, 0, sizeof(int32_t) * kPad, s));
+        AMG_CUDA(cudaMemsetAsync(P.v() + nnz, 0, sizeof(double) * kPad, s));
+    } else {
         TmpBuf prow(sizeof(int32_t) * (nnz + 1), s), coef(sizeof(double) * 3 * (size_t)n, s);
         { interp_rows_kernel<<<g, kThreads, 0, s>>>(n, A.rp(), A.ci(), A.v(), strong, cf, cmap, P.rp(), P.ci(),
-                                                  P.v(), prow.as<int32_t>(), coef.as<double>()); ::amg::count_launch(); }
+                                                  P.v(), prow.as<int32_t>(), coef.as<double>(), nnz); ::amg::count_launch(); }
         if (nnz > 0)
             { interp_weights_kernel<<<div_up(nnz, kThreads), kThreads, 0, s>>>(nnz, prow.as<int32_t>(),
                                                                              coef.as<double>(), P.v()); ::amg::count_launch(); }
@@ -2147,12 +2302,14 @@ void transpose(const DevCSR &M, DevCSR &T, cudaStream_t s) {
     T.nnz = nnz;
     T.col.alloc(sizeof(int32_t) * (nnz + kPad));
     T.val.alloc(sizeof(double) * (nnz + kPad));
-    AMG_CUDA(cudaMemsetAsync(T.ci() + nnz, 0, sizeof(int32_t) * kPad, s));  // the fill writes [0, nnz)
-    AMG_CUDA(cudaMemsetAsync(T.v() + nnz, 0, sizeof(double) * kPad, s));
+    if (M.nrows == 0) {  // no rows to move: the spare entries alone
+        AMG_CUDA(cudaMemsetAsync(T.ci() + nnz, 0, sizeof(int32_t) * kPad, s));
+        AMG_CUDA(cudaMemsetAsync(T.v() + nnz, 0, sizeof(double) * kPad, s));
+    }
     AMG_CUDA(cudaMemcpyAsync(fill.ptr, T.rp(), sizeof(int32_t) * (m + 1), cudaMemcpyDeviceToDevice, s));
     if (M.nrows > 0)
         { transpose_fill_kernel<<<div_up(M.nrows, kThreads), kThreads, 0, s>>>(
-            M.nrows, M.rp(), M.ci(), M.v(), fill.as<int32_t>(), T.ci(), T.v()); ::amg::count_launch(); }
+            M.nrows, M.rp(), M.ci(), M.v(), fill.as<int32_t>(), T.ci(), T.v(), nnz); ::amg::count_launch(); }
     if (m > 0) {
         const double mean = (double)nnz / (double)m;
         int W = 2;
@@ -2192,8 +2349,7 @@ static void spgemm_impl(const DevCSR &A, const SpRows &B, DevCSR &Cm, SlotProduc
         dcounts(sizeof(SpgemmCounts), s), cnt(sizeof(int32_t) * (n + 1), s), obase(sizeof(int64_t) * (n + 1), s);
     int g = div_up(n, kThreads);
     SpgemmCounts *dc = dcounts.as<SpgemmCounts>();
-    { spgemm_ub_kernel<<<g, kThreads, 0, s>>>(n, A.rp(), A.ci(), B.beg, B.end, ub.as<int64_t>()); ::amg::count_launch(); }
-    AMG_CUDA(cudaMemsetAsync(dcounts.ptr, 0, sizeof(SpgemmCounts), s));
+    { spgemm_ub_kernel<<<g, kThreads, 0, s>>>(n, A.rp(), A.ci(), B.beg, B.end, ub.as<int64_t>(), dc); ::amg::count_launch(); }
     { bin_rows_kernel<<<g, kThreads, 0, s>>>(n, ub.as<int64_t>(), bins.as<int32_t>(), dc); ::amg::count_launch(); }
     AMG_CHECK_LAUNCH();
     // product-bound offsets of the one-pass numeric kernel (total into the same record)
@@ -2354,9 +2510,7 @@ static void spgemm_impl(const DevCSR &A, const SpRows &B, DevCSR &Cm, SlotProduc
         Cm.nnz = nnz;
         Cm.col.alloc(sizeof(int32_t) * (nnz + kPad));
         Cm.val.alloc(sizeof(double) * (nnz + kPad));
-        AMG_CUDA(cudaMemsetAsync(Cm.ci() + nnz, 0, sizeof(int32_t) * kPad, s));
-        AMG_CUDA(cudaMemsetAsync(Cm.v() + nnz, 0, sizeof(double) * kPad, s));
-        { spgemm_compact_kernel<<<div_up((int64_t)n * kCompactLanes, 256), 256, 0, s>>>(n, obase.as<int64_t>(), Cm.rp(), tci.as<int32_t>(), tv.as<double>(), Cm.ci(), Cm.v()); ::amg::count_launch(); }
+        { spgemm_compact_kernel<<<div_up((int64_t)n * kCompactLanes, 256), 256, 0, s>>>(n, obase.as<int64_t>(), Cm.rp(), tci.as<int32_t>(), tv.as<double>(), Cm.ci(), Cm.v(), nnz); ::amg::count_launch(); }
         AMG_CHECK_LAUNCH();
         return;  // the temporaries' stream-ordered frees follow the compaction
     }
@@ -2491,12 +2645,13 @@ int64_t sparsify(const DevCSR &A, const uint8_t *inM, const int32_t *tpos, const
     H.nnz = nnz;
     H.col.alloc(sizeof(int32_t) * (nnz + kPad));
     H.val.alloc(sizeof(double) * (nnz + kPad));
-    AMG_CUDA(cudaMemsetAsync(H.ci() + nnz, 0, sizeof(int32_t) * kPad, s));  // the compaction writes [0, nnz)
-    AMG_CUDA(cudaMemsetAsync(H.v() + nnz, 0, sizeof(double) * kPad, s));
-    if (n > 0) {
+    if (n == 0) {  // no rows to compact: the spare entries alone
+        AMG_CUDA(cudaMemsetAsync(H.ci() + nnz, 0, sizeof(int32_t) * kPad, s));
+        AMG_CUDA(cudaMemsetAsync(H.v() + nnz, 0, sizeof(double) * kPad, s));
+    } else {
         if (full) {
             compact_values_kernel<<<g, kThreads, 0, s>>>(n, A.rp(), A.ci(), keep, hval.as<double>(), H.rp(), H.ci(),
-                                                        H.v());
+                                                        H.v(), nnz);
         } else {
             // at most 8 lanes a row: the lumped diagonal's additions are
             // issued by one lane per row, so a warp of one row would spend a
@@ -2504,7 +2659,7 @@ int64_t sparsify(const DevCSR &A, const uint8_t *inM, const int32_t *tpos, const
             with_row_lanes(std::min(row_lanes(A), 8), [&](auto tc) {
                 constexpr int L = decltype(tc)::value;
                 sparsify_compact_lanes_kernel<L><<<div_up((int64_t)n * L, kThreads), kThreads, 0, s>>>(
-                    n, A.rp(), A.ci(), A.v(), diagpos, keep, H.rp(), H.ci(), H.v());
+                    n, A.rp(), A.ci(), A.v(), diagpos, keep, H.rp(), H.ci(), H.v(), nnz);
             });
         }
         ::amg::count_launch();
