@@ -5,9 +5,8 @@
 // consecutive columns W t .. W t + W - 1, moved as one 16-byte vector (W = 4
 // floats or 2 doubles).  Every lane of the group reads the row's (column,
 // value) pairs itself -- the same address across the group, served as one
-// broadcast -- with the next kAhead entries' pairs on their way while the
-// vectors of this one's are gathered; each column sums its entries in row
-// order.  The matrix is read once per block of K right-hand sides instead of
+// broadcast -- kAhead entries at a time, their vector loads in flight
+// together; each column sums its entries in row order.  The matrix is read once per block of K right-hand sides instead of
 // K times.  A block takes a contiguous range of rows: what a row gathers of
 // the grid lines beside its own is then still in L1 from the block's last
 // steps, and L2 -- whose bandwidth bounds these kernels, a 7-point row at

@@ -1,7 +1,9 @@
 // cycle.cu -- V-cycle and PCG kernels.
 //
 // Every kernel here is a streaming pass over a sparse matrix or a few
-// vectors, so HBM bandwidth bounds it.  Two SpMV layouts serve all of them:
+// vectors: HBM bandwidth and the FP64 pipe (one warp instruction in 16 clocks
+// per SM) bound the large levels, a chain of dependent loads the small ones.
+// Three SpMV layouts serve all of them:
 //  * vector-CSR: a group of T lanes (T = 2..32) owns a row; each lane loads
 //    16-byte vectors of values and column indices (2 FP64 / 4 FP32 / 8 BF16
 //    entries) read through the non-coherent path, masks the entries outside
@@ -10,9 +12,12 @@
 //    warp with T = 32 / C lanes per row -- lane l takes row l % C and every
 //    T-th entry from l / C -- so each warp load is one contiguous
 //    128/256-byte segment whatever C; a shorter C splits long rows over more
-//    lanes (shorter dependent chains per thread) and pads less.
-// Reductions for PCG are deterministic: fixed grid, per-block partials, and
-// the last block to arrive sums them in block order.
+//    lanes (shorter dependent chains per thread) and pads less;
+//  * row patterns (patterns.cu), for a finest operator of few distinct rows:
+//    one byte a row, the rows themselves in shared memory.
+// Reductions for PCG are deterministic: fixed grid, per-block partials,
+// summed in block order by the last block to finish (small grids) or by a
+// one-block finisher kernel.
 #include <cuda_bf16.h>
 
 #include <cstdlib>
