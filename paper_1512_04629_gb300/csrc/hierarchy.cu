@@ -633,7 +633,13 @@ static bool prepare_level_at(Hierarchy &h, Level &V, int l, bool has_p, cudaStre
     // and read one lane per row in row order, as SELL-32: nothing to time.
     // Coarse operators are never that regular, and a forced variant is used
     // as given.  Below the tuning threshold a cycle is launch latency alone.
-    if (l == 0 && forced == AMG_SPMV_AUTO && M.nnz >= 20000 && has_p) {
+    // Long rows (more than 12 entries) on small grids stay with the lanes: one
+    // lane walking a row is then the kernel's time, not its bytes (27-point
+    // solves, general layouts / patterns, ms: 25^3 0.86 / 1.08, 28^3 0.98 /
+    // 0.99, 32^3 1.06 / 1.04, 36^3 1.25 / 1.14, 40^3 1.52 / 1.26).
+    constexpr int32_t kPatWideRows = 32768;
+    if (l == 0 && forced == AMG_SPMV_AUTO && M.nnz >= 20000 && has_p &&
+        (M.nnz <= 12 * (int64_t)M.nrows || M.nrows >= kPatWideRows)) {
         // temporaries until they are known to serve: a persistent buffer's
         // release would wait for the whole device, the coarsening included
         TmpBuf pid(n + kPad, s), tab(cyc::pat_table_bytes(), s);

@@ -40,14 +40,15 @@ CASES = {
     "2d5_71": (lambda: gen.poisson2d_5pt(71).to_scipy(), True),
     "2d5_96": (lambda: gen.poisson2d_5pt(96).to_scipy(), True),
     "3d7_17": (lambda: gen.poisson3d_7pt(17).to_scipy(), True),
-    "3d27_13": (lambda: gen.poisson3d_27pt(13).to_scipy(), True),
-    "q1_13": (lambda: gen.q1_laplace3d(13).to_scipy(), True),
+    "3d27_13": (lambda: gen.poisson3d_27pt(13).to_scipy(), False),  # long rows, few of them
+    "3d27_33": (lambda: gen.poisson3d_27pt(33).to_scipy(), True),
+    "q1_33": (lambda: gen.q1_laplace3d(33).to_scipy(), True),
     "aniso_67": (lambda: gen.rotated_aniso_q1(67).to_scipy(), True),
     "one_row_short_of_a_block": (lambda: _classes(8191, 3), True),
     "most_patterns": (lambda: _classes(8000, 253), True),
     "one_pattern_too_many": (lambda: _classes(8000, 254), False),
-    "longest_row": (lambda: _band(1500, 15), True),
-    "rows_too_long": (lambda: _band(1500, 16), False),
+    "longest_row": (lambda: _band(32800, 15), True),
+    "rows_too_long": (lambda: _band(32800, 16), False),
     "lognormal": (lambda: gen.fv7_lognormal(17, seed=3).to_scipy(), False),
 }
 
