@@ -28,6 +28,9 @@ Also reported, all outside the timed region:
   * `cpu_baseline`: the CPU oracle on every host core (its all-core build:
     the solve phase's loops under OpenMP, setup sequential), with the
     sequential build's figure beside it.
+Standard output gets one short line: the headline, what qualifies it, and one
+figure per arm and leg.  The full record goes to `--details FILE`, or to
+standard error.
 `--impl reference` times the all-core CPU oracle on the same workload.
 """
 from __future__ import annotations
@@ -89,6 +92,9 @@ def parse():
                         "(Algorithm 3)")
     p.add_argument("--krylov", default="cg", choices=["cg", "gmres"],
                    help="outer solver: PCG (default) or restarted GMRES(30)")
+    p.add_argument("--details", default=None, metavar="FILE",
+                   help="write the full record of the default workload (every kernel, level, arm and leg) to FILE "
+                        "instead of to standard error")
     p.add_argument("--eager", action="store_true",
                    help="launch the PCG iterations one kernel at a time (no CUDA graph; for ncu launch lists)")
     p.add_argument("--ncu-setup", action="store_true",
@@ -799,6 +805,52 @@ def solve_arms(args, A_dev, nnz0, bd, xd, stream, reps=5):
     return arms
 
 
+def _short(x):
+    """x with every float cut to six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_short(v) for v in x]
+    return x
+
+
+def headline(full):
+    """The line printed on standard output: the result with what qualifies it
+    (configuration, clocks, roofline, end to end, baseline) and one figure per
+    arm and leg.  Readers keep the last few thousand characters of a run's
+    output, so the whole record (20 KB) goes elsewhere and this stays below
+    2,800 characters."""
+    out = {k: full[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "iterations")}
+    roof = full["roofline"]
+    out["roofline"] = {k: roof[k] for k in ("kernel", "bound", "achieved", "peak", "unit", "frac", "traffic",
+                                            "algorithmic_bytes_per_launch", "avg_launch_ms")}
+    if "fp64" in roof:
+        out["roofline"]["fp64_frac"] = roof["fp64"]["frac"]
+    out["vcycle_GBps"] = full["vcycle_GBps"]
+    out["e2e"] = full["e2e"]
+    cpu = full["cpu_baseline"]
+    out["cpu_baseline"] = cpu and {k: cpu[k] for k in ("value", "unit", "cores", "kind")}
+    arms = full["arms"]
+    out["arms_ms"] = arms and {k: v["time_to_tol_ms"] for k, v in arms.items()}
+    legs = {}
+    for name, leg in (full["legs"] or {}).items():
+        if "error" in leg:
+            legs[name] = {"error": leg["error"][:80]}
+        elif "arms" in leg:  # milliseconds per arm
+            legs[name] = {k: v["time_to_tol_ms"] if "time_to_tol_ms" in v else v["ms"] for k, v in leg["arms"].items()}
+        else:
+            legs[name] = {k: leg[k] for k in ("requests", "failed", "solves_per_s", "p50_ms", "p99_ms")}
+        if leg.get("clocks"):
+            legs[name]["sm_mhz"] = leg["clocks"]["sm_mhz"]
+    out["legs"] = legs or None
+    out["clocks"] = full["clocks"]
+    out["gpu_launches"] = full["gpu_launches"]
+    return dict(_short(out), value=full["value"], ms_per_step=full["ms_per_step"])
+
+
 def main():
     args = parse()
     if args.impl == "reference":
@@ -1051,7 +1103,13 @@ def main():
         "e2e": e2e, "cpu_baseline": cpu, "arms": arms, "communication": comm, "legs": legs, "clocks": clocks,
         "gpu_launches": launches,
     }
-    print(json.dumps(line))
+    details = json.dumps(line)
+    if args.details:
+        with open(args.details, "w") as f:
+            f.write(details + "\n")
+    else:
+        print(details, file=sys.stderr, flush=True)
+    print(json.dumps(headline(line)))
     if dist:
         dist.barrier()
         dist.destroy_process_group()
