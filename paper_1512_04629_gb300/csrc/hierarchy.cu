@@ -1406,12 +1406,21 @@ void ensure_graph(Hierarchy &h) {
     h.graph_dirty = false;
 }
 
-// A run of at most this many steps (a window of Algorithm 5) on a hierarchy
-// that has changed since its graph was built is launched kernel by kernel:
-// nearly every window ends in a reintroduction, and capturing and
-// instantiating the step costs what several eager steps do (adaptive solves
-// from gamma = 1, windows of 3: 75^3 9.5 -> 8.4 ms, 128^3 21.3 -> 19.9 ms).
+// The first run of at most this many steps (a window of Algorithm 5) on a
+// hierarchy that has changed is launched kernel by kernel: when windows end in
+// reintroductions, capturing and instantiating the step for each of them costs
+// what several such steps do (adaptive solves from gamma = 1, windows of 3:
+// 75^3 9.5 -> 8.4 ms, 128^3 21.3 -> 19.9 ms).  A second run on the same
+// version gets its graph, and so do all that follow.
 constexpr int kEagerSteps = 4;
+
+// Whether a run of max_steps steps on a hierarchy without a current graph
+// goes without one; notes it, so that the next one does not.
+bool run_eager(Hierarchy &h, int max_steps) {
+    if (max_steps > kEagerSteps || h.eager_version == h.version) return false;
+    h.eager_version = h.version;
+    return true;
+}
 
 // Runs up to max_steps CG steps (stopping at the recurrence test, then
 // confirming with the true residual; a failed confirmation replaces r).
@@ -1425,7 +1434,8 @@ void pcg_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int ma
     run = Run();
     run.rnorm = rnorm_now;
     if (rnorm_now <= tol * bnorm) { run.converged = true; return; }
-    bool graph = h.opt.use_graph && !h.timing && !(max_steps <= kEagerSteps && h.graph_dirty);
+    bool graph = h.opt.use_graph && !h.timing;
+    if (graph && h.graph_dirty && run_eager(h, max_steps)) graph = false;
     if (graph) ensure_graph(h);
     double thresh2 = (tol * bnorm) * (tol * bnorm);
     int32_t n = h.lev[0]->n();
@@ -1623,7 +1633,8 @@ void gm_iterate(Hierarchy &h, const double *b, double bnorm, double tol, int max
     GmresScalars &c = *h.h_gsc;
     run.rnorm = c.est;
     if (c.est <= thresh) { run.converged = true; return; }
-    const bool graph = h.opt.use_graph && !h.timing && !(max_steps <= kEagerSteps && h.g_gmres_version != h.version);
+    bool graph = h.opt.use_graph && !h.timing;
+    if (graph && h.g_gmres_version != h.version && run_eager(h, max_steps)) graph = false;
     if (graph) gm_ensure_graph(h);
     while (run.steps < max_steps) {
         if (c.j == h.gm_m) {  // restart
