@@ -1406,20 +1406,25 @@ void ensure_graph(Hierarchy &h) {
     h.graph_dirty = false;
 }
 
-// The first run of at most this many steps (a window of Algorithm 5) on a
-// hierarchy that has changed is launched kernel by kernel: when windows end in
-// reintroductions, capturing and instantiating the step for each of them costs
-// what several such steps do (adaptive solves from gamma = 1, windows of 3:
-// 75^3 9.5 -> 8.4 ms, 128^3 21.3 -> 19.9 ms).  A second run on the same
-// version gets its graph, and so do all that follow.
-constexpr int kEagerSteps = 4;
+// The first kEagerRuns runs of at most kEagerSteps steps (windows of Algorithm
+// 5) on a hierarchy that has changed are launched kernel by kernel: when
+// windows end in reintroductions, capturing and instantiating the step for
+// each of them costs what several such steps do (adaptive solves from gamma =
+// 1, windows of 3: 75^3 9.5 -> 8.4 ms, 128^3 21.3 -> 19.9 ms).  The next run on
+// the same version gets its graph, and so do all that follow.  With one such
+// run instead of two the solves that end soon after their last reintroduction
+// pay for a graph that they use once (75^3: 8.6 ms).
+constexpr int kEagerSteps = 4, kEagerRuns = 2;
 
 // Whether a run of max_steps steps on a hierarchy without a current graph
-// goes without one; notes it, so that the next one does not.
+// goes without one; counts it.
 bool run_eager(Hierarchy &h, int max_steps) {
-    if (max_steps > kEagerSteps || h.eager_version == h.version) return false;
-    h.eager_version = h.version;
-    return true;
+    if (max_steps > kEagerSteps) return false;
+    if (h.eager_version != h.version) {
+        h.eager_version = h.version;
+        h.eager_runs = 0;
+    }
+    return h.eager_runs++ < kEagerRuns;
 }
 
 // Runs up to max_steps CG steps (stopping at the recurrence test, then

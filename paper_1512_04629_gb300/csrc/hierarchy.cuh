@@ -162,7 +162,7 @@ struct Hierarchy {
     cudaStream_t graph_stream = nullptr;
     bool graph_dirty = true;
     int version = 0;  // bumped whenever the cycle's buffers or operators change
-    int eager_version = -1;  // the version on which a short run went without a graph
+    int eager_version = -1, eager_runs = 0;  // short runs without a graph on that version
 
     std::map<int, std::unique_ptr<BatchWS>> batch;
 
