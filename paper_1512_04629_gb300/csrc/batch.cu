@@ -102,19 +102,30 @@ __device__ __forceinline__ void entries(int32_t e, const int32_t *__restrict__ c
 // acc += sum over the row's entries, in entry order, of a_ij * src_j[c0 ..]
 // (SCALE: times dinv_j, for x_j = dinv_j b_j that was never written); SUB:
 // subtracted, for residuals whose accumulator starts at b.  kAhead entries
-// at a time, the rest by halves -- no predicated-off FMAs, which would cost
-// the FP64 pipe as much as real ones
+// at a time, the rest by halves.  In FP64 the rest is written as loops, which
+// the compiler leaves as branches: as plain conditions it predicates them,
+// and a predicated-off FMA holds the FP64 pipe like a real one -- in A p over
+// rows of five entries (4 + 1) the two absent ones took 501 us instead of 399
+// at 2D 2048^2, K = 8.  In FP32 conditions are the faster form (lognormal
+// 112^3, K = 32: 0.8% of the solve).
 template <typename VT, typename XT, int K, bool SCALE, bool SUB>
 __device__ __forceinline__ void row_block_sum(int32_t p0, int32_t p1, const int32_t *__restrict__ ci,
                                               const VT *__restrict__ v, const XT *__restrict__ src,
                                               const XT *__restrict__ dinv, int c0, XT (&acc)[16 / sizeof(XT)]) {
     int32_t e = p0;
     for (; e + kAhead <= p1; e += kAhead) entries<kAhead, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
-    if (e + 2 <= p1) {
-        entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
-        e += 2;
+    if constexpr (sizeof(XT) == 8) {
+#pragma unroll 1
+        for (; e + 2 <= p1; e += 2) entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+#pragma unroll 1
+        for (; e < p1; ++e) entries<1, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+    } else {
+        if (e + 2 <= p1) {
+            entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
+            e += 2;
+        }
+        if (e < p1) entries<1, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
     }
-    if (e < p1) entries<1, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
 }
 
 // operands of an SpMM pass (unused ones null)
