@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "batch_ops.cuh"
@@ -303,15 +304,23 @@ col_finish_kernel(int nblocks, const double *partials, ColScalars sc, int flexib
     }
 }
 
-// at least four rows per thread and at most one resident wave of blocks
-int grid_for(int64_t n, int K) {
-    int64_t rows_per_block = kThreads / K;
-    int64_t b = (n + rows_per_block - 1) / rows_per_block;
-    b = (b + 3) / 4;
-    int64_t cap = std::min<int64_t>(kBatchReduceBlocks, ::amg::resident_blocks(kThreads));
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    return (int)b;
+// Blocks of a reducing kernel that gives each row G lanes: one resident wave,
+// at least four rows per lane group.  The wave is asked of the runtime: with
+// eight blocks per SM assumed, r.z of FP32 cycles, whose 42 registers let five
+// stay, ran in two waves, the second three fifths full (2D 2048^2, K = 8: 178
+// us, 129 as one wave).
+template <auto KERN> int reduce_grid(int32_t n, int G) {
+    static std::atomic<int> per_sm{0};
+    int b = per_sm.load(std::memory_order_relaxed);
+    if (b == 0) {
+        AMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, KERN, kThreads, 0));
+        b = std::max(b, 1);
+        per_sm.store(b, std::memory_order_relaxed);
+    }
+    const int64_t rows = kThreads / G;
+    const int64_t want = ((n + rows - 1) / rows + 3) / 4;
+    const int64_t cap = std::min<int64_t>(kBatchReduceBlocks, (int64_t)b * ::amg::resident_blocks(2048));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
 }
 
 __device__ __forceinline__ void zload(const double *p, double (&z)[2]) { vload(p, z); }
@@ -586,8 +595,9 @@ template <typename ZT>
 void rz(int32_t n, int K, const double *R, const ZT *Z, const double *Q, ColScalars sc, double *partials,
         cudaStream_t s) {
     constexpr int NV = sizeof(ZT) == 8 ? 1 : 2;  // FP32 cycles: flexible CG, whose beta needs z.q
-    const int blocks = grid_for(n, K / 2);
+    int blocks = 0;
     with_width(K, [&](auto kc) {
+        blocks = reduce_grid<rz_kernel<decltype(kc)::value, NV, ZT>>(n, K / 2);
         rz_kernel<decltype(kc)::value, NV, ZT><<<blocks, kThreads, 0, s>>>(n, R, Z, Q, partials);
         ::amg::count_launch();
     });
@@ -603,25 +613,10 @@ template <typename ZT> void p_update(int32_t n, int K, const ZT *Z, double *P, C
     });
 }
 
-// one resident wave of ap_kernel blocks (at least four rows per thread group)
-template <int K, bool RESID>
-static int ap_grid(int32_t n) {
-    static int per_sm = 0;
-    if (per_sm == 0) {
-        int b = 0;
-        AMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, ap_kernel<K, RESID>, kThreads, 0));
-        per_sm = std::max(b, 1);
-    }
-    const int64_t rpb = kThreads / (K / 2);
-    const int64_t want = ((n + rpb - 1) / rpb + 3) / 4;
-    const int64_t cap = std::min<int64_t>(kBatchReduceBlocks, (int64_t)per_sm * ::amg::resident_blocks(2048));
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, cap));
-}
-
 template <int K, bool RESID>
 static void launch_ap_k(const CycMat<double> &A, const double *P, const double *B, double *Q, ColScalars sc,
                         double *partials, cudaStream_t s) {
-    const int blocks = ap_grid<K, RESID>(A.nrows);
+    const int blocks = reduce_grid<ap_kernel<K, RESID>>(A.nrows, K / 2);
     { ap_kernel<K, RESID><<<blocks, kThreads, 0, s>>>(A.nrows, A.rp, A.ci, A.v, P, B, Q, partials); ::amg::count_launch(); }
     if (RESID) { col_finish_kernel<1, kColTt><<<K, kThreads, 0, s>>>(blocks, partials, sc, 0); ::amg::count_launch(); }
     else { col_finish_kernel<1, kColAp><<<K, kThreads, 0, s>>>(blocks, partials, sc, 0); ::amg::count_launch(); }
@@ -652,8 +647,9 @@ void residual(const CycMat<double> &A, int K, const double *B, const double *X, 
 
 void xr_update(int32_t n, int K, const double *P, const double *Q, double *X, double *R, float *R32, ColScalars sc,
                double *partials, cudaStream_t s) {
-    const int blocks = grid_for(n, K / 2);
+    int blocks = 0;
     with_width(K, [&](auto kc) {
+        blocks = reduce_grid<xr_kernel<decltype(kc)::value>>(n, K / 2);
         xr_kernel<decltype(kc)::value><<<blocks, kThreads, 0, s>>>(n, P, Q, X, R, R32, sc, partials);
         ::amg::count_launch();
     });
