@@ -6,16 +6,17 @@
 // floats or 2 doubles).  Every lane of the group reads the row's (column,
 // value) pairs itself -- the same address across the group, served as one
 // broadcast -- kAhead entries at a time, their vector loads in flight
-// together; each column sums its entries in row order.  The matrix is read once per block of K right-hand sides instead of
-// K times.  A block takes a contiguous range of rows: what a row gathers of
-// the grid lines beside its own is then still in L1 from the block's last
-// steps, and L2 -- whose bandwidth bounds these kernels, a 7-point row at
-// K = 32 gathers 7 x 128 bytes -- serves it about once instead of per row.
-// Lognormal 112^3, K = 32, FP32, finest level: residual 165 -> 113 us (it no
-// longer writes x = D^-1 b either), prolongation 124 -> 97, post-smoothing
-// 170 -> 121 (it writes the correction in FP32, not widened); the whole
-// solve 78.3 -> 73.0 ms.  Forming r.z in the post-smoothing too was slower
-// (340 us against 121 + 179): its registers leave half the warps.
+// together; each column sums its entries in row order.  The matrix is read
+// once per block of K right-hand sides instead of K times.  A block takes a
+// contiguous range of rows: what a row gathers of the grid lines beside its
+// own is then still in L1 from the block's last steps, and L2 -- whose
+// bandwidth bounds these kernels, a 7-point row at K = 32 gathers 7 x 128
+// bytes -- serves it about once instead of per row (how long a range:
+// spmm_grid).  Lognormal 112^3, K = 32, FP32, finest level: residual 165 ->
+// 113 us (it no longer writes x = D^-1 b either), prolongation 124 -> 97,
+// post-smoothing 170 -> 121 (it writes the correction in FP32, not widened).
+// Forming r.z in the post-smoothing too was slower (340 us against 121 + 179):
+// its registers leave half the warps.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -190,9 +191,23 @@ spmm_kernel(int32_t n, int32_t chunk, const int32_t *__restrict__ rp, const int3
     }
 }
 
-// A block's threads and rows: as many blocks as stay resident, each with an
-// even contiguous share; levels too small to fill the device that way get
-// smaller blocks, down to one warp's rows each.
+// A block's threads and rows.  Blocks take ranges of about kSpmmSteps steps
+// (64 KB of the gathered block), in as many even waves as that makes: blocks
+// start in order, so the rows at work at one time are a front that moves
+// through the matrix, and what a row gathers a grid plane away is in L2 from
+// the front's last pass or about to serve its next.  With one range per
+// resident block over the whole matrix that neighbour lies in another block's
+// range, and above the L2's size it comes from HBM again; such a pass also
+// holds the whole device for its time, and the short passes of other
+// hierarchies wait.  Solves in ms, whole-matrix ranges -> these: lognormal,
+// K = 64, 96^3 86.3 -> 83.0, 112^3 136.7 -> 137.1, 128^3 242 -> 228, 160^3
+// 535 -> 485; K = 32, 112^3 73.0 -> 74.0, 128^3 124.3 -> 118.6, 160^3 270 ->
+// 251; 2D 2048^2, K = 8 109.5 -> 104.7.  Ranges of 4 or 6 steps are within 1%
+// of 8, of 16 and 32 up to 6% slower, of 1 (rows in launch order) 7-10%.
+// Serving eight hierarchies, p50 / p99: 99 / 299 -> 88 / 235 ms.  Levels
+// that fill the device less than once get smaller blocks, down to one warp's
+// rows each.
+constexpr int kSpmmSteps = 8;
 struct SpmmGrid {
     int threads, blocks;
     int32_t chunk;
@@ -204,7 +219,8 @@ SpmmGrid spmm_grid(int64_t n, int G, int resident) {
     const int64_t rows = threads / G;  // per step
     const int64_t want = (n + rows - 1) / rows;
     const int64_t cap = sms * resident * (kSpmmThreads / threads);
-    const int64_t steps = (want + cap - 1) / cap;
+    const int64_t waves = std::max<int64_t>(1, (want + cap - 1) / cap / kSpmmSteps);
+    const int64_t steps = (want + cap * waves - 1) / (cap * waves);
     SpmmGrid g;
     g.threads = threads;
     g.chunk = (int32_t)(steps * rows);
