@@ -393,8 +393,12 @@ __global__ void pmis_apply_kernel(const int32_t *list, const int *len, int32_t n
 // in launches -> in one block (median ms): 32 x 32 1.62 -> 1.47, 45 x 45
 // 1.77 -> 1.62, 101 x 101 2.26 -> 2.10, 128^3 9.68 -> 9.61.  With the line at
 // 1024 rows the 45 x 45 one takes 1.69; at 4096 the 101 x 101 one 2.20 and the
-// 128^3 one 10.0.
+// 128^3 one 10.0.  A sweep also walks every entry, on one SM, so levels of many
+// entries stay with the launches: 2000 rows of 38 entries 1.68 -> 1.65 ms, of 76
+// 1.79 -> 1.91, of 150 2.17 -> 2.38, of 298 4.97 -> 5.92; 1000 rows of 60 1.43 ->
+// 1.35, of 221 2.80 -> 2.91.
 constexpr int kPmisSmall = 2048, kPmisThreads = 1024;
+constexpr int64_t kPmisSmallEntries = 100000;
 template <int T>
 __global__ void __launch_bounds__(kPmisThreads)
 pmis_small_kernel(int32_t n, const int32_t *rp, const int32_t *ci, const int32_t *tpos, const uint8_t *strong,
@@ -2139,7 +2143,7 @@ int64_t pmis(const DevCSR &A, const uint8_t *strong, const int32_t *tpos, uint64
         return 0;
     }
     const int T = row_lanes(A, 8);
-    if (n <= kPmisSmall) {
+    if (n <= kPmisSmall && A.nnz <= kPmisSmallEntries) {
         TmpBuf sym(A.nnz + 1, s), out(2 * sizeof(int), s);
         with_row_lanes(T, [&](auto tc) {
             constexpr int L = decltype(tc)::value;
