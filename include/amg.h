@@ -148,7 +148,7 @@ typedef struct {
     double gamma;           /* drop tolerance of the level */
     int spmv_variant;       /* AMG_SPMV_* used by the level's relaxation */
     int value_bytes;        /* bytes per stored value in the cycle (8, 4, 2) */
-    double bytes_per_cycle; /* algorithmic HBM bytes of the level per V(1,1) cycle */
+    double bytes_per_cycle; /* algorithmic HBM bytes of the level per V(1,1) cycle (as amg_timing_get) */
     int spmv_variant_p;     /* AMG_SPMV_* of the interpolation x += P x_c (0 on the coarsest) */
     int spmv_variant_r;     /* AMG_SPMV_* of the restriction b_c = R r (0 on the coarsest) */
 } amg_level_info;
@@ -261,7 +261,9 @@ amg_status amg_level_array(const amg_hierarchy *h, int level, int which, void *o
  * amg_timing_get returns, for kernel class `kind` (0 fused pre-smooth +
  * residual, 1 restrict, 2 prolong, 3 post-smooth, 4 coarse solve, 5 PCG
  * A p + dot, 6 PCG vector update) on `level`, the number of timed launches,
- * their total milliseconds and their algorithmic bytes.  With
+ * their total milliseconds and their algorithmic bytes (operators as CSR
+ * arrays; a finest operator stored by its distinct rows as those and one byte
+ * per row).  With
  * amg_options.setup_timing, or while timing is enabled during amg_sparsify /
  * amg_reintroduce, the setup phases are recorded too (bytes 0): 8 strength,
  * 9 C/F splitting (PMIS and the coarse numbering), 10 interpolation P and

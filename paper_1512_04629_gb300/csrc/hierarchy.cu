@@ -1104,22 +1104,28 @@ void ensure_workspace(Hierarchy &h, cudaStream_t s) {
 // ---------------------------------------------------------------------------
 // algorithmic bytes (compulsory HBM traffic) per kernel launch
 // ---------------------------------------------------------------------------
-static double bytes_pre(int64_t n, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (n + 1) + 4.0 * n * xb; }
+// an operator of vb-byte values: its CSR arrays, or, stored by row patterns, one
+// byte per row and the table
+static double bytes_csr(int64_t n, int64_t nnz, int vb) { return (double)nnz * (vb + 4) + 4.0 * (n + 1); }
+static double bytes_op(const Level &V, int vb) {
+    if (V.npat > 0 && !V.part_h) return (double)V.n() + (double)V.npat * (V.pwidth + 1) * (vb + 4);
+    return bytes_csr(V.n(), V.op().nnz, vb);
+}
+static double bytes_pre(const Level &V, int xb) { return bytes_op(V, V.vbytes) + 4.0 * V.n() * xb; }
 // levels >= 1: x = D^{-1} b was written by the restriction; read b, x, write r
-static double bytes_pre_x(int64_t n, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (n + 1) + 3.0 * n * xb; }
+static double bytes_pre_x(const Level &V, int xb) { return bytes_op(V, V.vbytes) + 3.0 * V.n() * xb; }
 // restriction that also writes the coarse pre-smooth x_c = d_c .* b_c
-static double bytes_restrict_x(int64_t nc, int64_t n, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (nc + 1) + (double)(n + 3 * nc) * xb; }
-static double bytes_post(int64_t n, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (n + 1) + 4.0 * n * xb; }
-static double bytes_restrict(int64_t nc, int64_t n, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (nc + 1) + (double)(n + nc) * xb; }
-static double bytes_prolong(int64_t n, int64_t nc, int64_t nnz, int vb, int xb) { return (double)nnz * (vb + 4) + 4.0 * (n + 1) + (double)(nc + 2 * n) * xb; }
+static double bytes_restrict_x(int64_t nc, int64_t n, int64_t nnz, int vb, int xb) { return bytes_csr(nc, nnz, vb) + (double)(n + 3 * nc) * xb; }
+static double bytes_post(const Level &V, int xb) { return bytes_op(V, V.vbytes) + 4.0 * V.n() * xb; }
+static double bytes_restrict(int64_t nc, int64_t n, int64_t nnz, int vb, int xb) { return bytes_csr(nc, nnz, vb) + (double)(n + nc) * xb; }
+static double bytes_prolong(int64_t n, int64_t nc, int64_t nnz, int vb, int xb) { return bytes_csr(n, nnz, vb) + (double)(nc + 2 * n) * xb; }
 
 double level_cycle_bytes(const Hierarchy &h, int l) {
     const Level &V = *h.lev[l];
     int xb = h.opt.precision == AMG_PREC_FP64 ? 8 : 4;
-    int64_t n = V.n(), nnz = V.op().nnz;
+    int64_t n = V.n();
     if (l == h.nlev() - 1) return (double)n * n * 8 + 2.0 * n * xb;
-    double b = (l == 0 ? bytes_pre(n, nnz, V.vbytes, xb) : bytes_pre_x(n, nnz, V.vbytes, xb)) +
-               bytes_post(n, nnz, V.vbytes, xb);
+    double b = (l == 0 ? bytes_pre(V, xb) : bytes_pre_x(V, xb)) + bytes_post(V, xb);
     b += (l + 2 < h.nlev() ? bytes_restrict_x(V.R.nrows, n, V.R.nnz, xb, xb) : bytes_restrict(V.R.nrows, n, V.R.nnz, xb, xb)) +
          bytes_prolong(n, V.P.ncols, V.P.nnz, xb, xb);
     return b;
@@ -1137,7 +1143,7 @@ template <typename XT>
 static void relax_pre(Hierarchy &h, int l, const XT *b, cudaStream_t s, bool x_ready) {
     Level &V = *h.lev[l];
     int xb = sizeof(XT);
-    const double bytes = x_ready ? bytes_pre_x(V.n(), V.op().nnz, V.vbytes, xb) : bytes_pre(V.n(), V.op().nnz, V.vbytes, xb);
+    const double bytes = x_ready ? bytes_pre_x(V, xb) : bytes_pre(V, xb);
     timed(h, 0, l, bytes, s, [&] {
         if (!x_ready) cyc::scale<XT>(V.n(), b, dinv_of<XT>(V), V.x.as<XT>(), s);
         if constexpr (sizeof(XT) == 8) {
@@ -1155,7 +1161,7 @@ template <typename XT>
 static void relax_post(Hierarchy &h, int l, const XT *b, XT *out, cudaStream_t s) {
     Level &V = *h.lev[l];
     int xb = sizeof(XT);
-    timed(h, 3, l, bytes_post(V.n(), V.op().nnz, V.vbytes, xb), s, [&] {
+    timed(h, 3, l, bytes_post(V, xb), s, [&] {
         if constexpr (sizeof(XT) == 8) {
             cyc::post_smooth<double, double>(op_mat<double>(V), V.x.as<XT>(), b, dinv_of<XT>(V), out, s);
         } else {
@@ -1204,7 +1210,7 @@ static bool vcycle_impl(Hierarchy &h, const XT *b0, XT *z0, cudaStream_t s, cons
             if (l == 0 && ctl.fuse_rz && V.vbytes == 8) {
                 // z.q only for flexible CG (plain CG's beta is r.z / rho)
                 const double *q = h.opt.precision != AMG_PREC_FP64 ? ctl.q : nullptr;
-                timed(h, 3, 0, bytes_post(V.n(), V.op().nnz, V.vbytes, xb) + (q ? 8.0 * V.n() : 0.0), s, [&] {
+                timed(h, 3, 0, bytes_post(V, xb) + (q ? 8.0 * V.n() : 0.0), s, [&] {
                     fused = cyc::post_smooth_rz(op_mat<double>(V), V.x.as<double>(), b, dinv_of<double>(V), z0, q,
                                                 h.dscal(), h.reduce(), s);
                 });
@@ -1328,7 +1334,7 @@ void pcg_start(Hierarchy &h, cudaStream_t s) {
 void pcg_body(Hierarchy &h, cudaStream_t s, cudaGraphConditionalHandle handle, bool use_handle) {
     int32_t n = h.lev[0]->n();
     CycMat<double> A0 = a0_mat(h);
-    double ap_bytes = (double)A0.nnz * 12 + 4.0 * (n + 1) + 16.0 * n;
+    double ap_bytes = bytes_op(*h.lev[0], 8) + 16.0 * n;
     CycleCtl ctl;
     ctl.x0_ready = true;  // pcg_start / replacement / the previous x, r update formed it
     ctl.fuse_rz = true;
@@ -1550,7 +1556,7 @@ void gm_step(Hierarchy &h, cudaStream_t s, cudaGraphConditionalHandle handle, bo
     vcycle_f64(h, h.pr.as<double>(), h.pz.as<double>(), s, ctl);
     timed(h, 6, 0, 16.0 * n, s, [&] { gm::store_z(n, h.pz.as<double>(), Z, sc, s); });
     CycMat<double> A0 = a0_mat(h);
-    const double ap_bytes = (double)A0.nnz * 12 + 4.0 * (n + 1) + 16.0 * n;
+    const double ap_bytes = bytes_op(*h.lev[0], 8) + 16.0 * n;
     timed(h, 5, 0, ap_bytes, s, [&] { cyc::spmv<double, double>(A0, h.pz.as<double>(), w, false, s); });
     timed(h, 6, 0, 0.0, s, [&] {
         gm::mdot(n, m, V, w, sc, ar, false, s);
