@@ -915,8 +915,8 @@ void launch_finish(int nblocks, Reduce red, PcgScalars *sc, cudaStream_t s, cons
 }
 
 // Grid of a reducing kernel: at most one resident wave, so every thread
-// loops over several rows and the shuffle tree of the block reduction (FP64
-// adds, the scarce pipe on this part) runs once per thread, not once per row.
+// loops over several rows and the block's reduction (FP64 adds, the scarce
+// pipe on this part) runs once per thread, not once per row.
 int reduce_blocks(int64_t threads_needed) {
     int64_t b = (threads_needed + kThreads - 1) / kThreads;
     int64_t cap = ::amg::resident_blocks(kThreads);
@@ -925,7 +925,6 @@ int reduce_blocks(int64_t threads_needed) {
     if (b < 1) b = 1;
     return (int)b;
 }
-static_assert(kThreads == 256, "two-level reduction assumes groups of 256 blocks and 256 threads");
 
 // ---------------------------------------------------------------------------
 // PCG kernels (FP64)

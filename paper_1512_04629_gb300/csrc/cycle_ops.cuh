@@ -88,11 +88,11 @@ struct PcgScalars {
     int pad;
 };
 
-// Deterministic reduction workspace: per-block partials + arrival counter.
+// Deterministic reduction workspace: one partial per block and value, and the
+// count of blocks done of a kernel that finishes itself (zero between kernels).
 struct Reduce {
-    double *partials = nullptr;   // 4 * kMaxReduceBlocks (per block)
-    unsigned *counter = nullptr;  // [0]: groups done; [1 + g]: blocks done in group g (257 used)
-    double *gpartials = nullptr;  // 4 * 256 (per group of 256 blocks)
+    double *partials = nullptr;   // 4 * kMaxReduceBlocks
+    unsigned *counter = nullptr;
 };
 constexpr int kMaxReduceBlocks = 65536;
 

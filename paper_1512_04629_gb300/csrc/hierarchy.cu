@@ -1094,8 +1094,8 @@ void ensure_workspace(Hierarchy &h, cudaStream_t s) {
     }
     h.scal.alloc(sizeof(PcgScalars));
     AMG_CUDA(cudaMemsetAsync(h.scal.ptr, 0, sizeof(PcgScalars), s));
-    h.partials.alloc(sizeof(double) * (4 * kMaxReduceBlocks + 4 * 256));
-    h.counter.alloc(sizeof(unsigned) * 512);
+    h.partials.alloc(sizeof(double) * 4 * kMaxReduceBlocks);
+    h.counter.alloc(sizeof(unsigned));
     AMG_CUDA(cudaMemsetAsync(h.counter.ptr, 0, h.counter.bytes, s));
     if (!h.h_scal) AMG_CUDA(cudaMallocHost(&h.h_scal, sizeof(PcgScalars)));
     h.ws_n = n;

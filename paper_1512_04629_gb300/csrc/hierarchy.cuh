@@ -179,7 +179,7 @@ struct Hierarchy {
     ~Hierarchy();
     int nlev() const { return (int)lev.size(); }
     Reduce reduce() {
-        return Reduce{partials.as<double>(), counter.as<unsigned>(), partials.as<double>() + 4 * kMaxReduceBlocks};
+        return Reduce{partials.as<double>(), counter.as<unsigned>()};
     }
     PcgScalars *dscal() { return scal.as<PcgScalars>(); }
 };
