@@ -69,11 +69,12 @@ void batch_push_flags(BatchWS &w, cudaStream_t s) {
     AMG_CUDA(cudaMemcpyAsync(w.sc.active, w.h_i, sizeof(int) * 2 * w.K, cudaMemcpyHostToDevice, s));
 }
 
-// Z = M B0 over the hierarchy's levels (at least two).  The FP32 cycle never writes a pre-smooth x = D^{-1} b: the residual multiplies by
-// D^{-1} as it gathers and the prolongation forms x from b.  In FP64 that
-// multiplication would double the passes' work on the FP64 pipe, which bounds
-// them, so x is written there -- with the restriction, or by a pass of its own
-// on the finest level.
+// Z = M B0 over the hierarchy's levels (at least two).  The FP32 cycle never
+// writes a pre-smooth x = D^{-1} b: the residual multiplies by D^{-1} as it
+// gathers and the prolongation forms x from b.  In FP64 that multiplication
+// would double the passes' work on the FP64 pipe, which bounds them, so x is
+// written there -- with the restriction, or by a pass of its own on the finest
+// level.
 template <typename XT>
 static void batch_vcycle_impl(Hierarchy &h, BatchWS &w, const XT *B0, XT *Z0, cudaStream_t s) {
     constexpr bool kF64 = sizeof(XT) == 8;

@@ -205,10 +205,7 @@ __device__ __forceinline__ XT sell_row_sum(int32_t pos, int32_t row, const int32
 // A p 391 -> 327 (304).  Six resident blocks per SM: with five the 27-point
 // solve takes 25.2 ms instead of 23.6, with eight (32 registers) 23.8.
 // ---------------------------------------------------------------------------
-#ifndef AMG_PAT_BLOCKS
-#define AMG_PAT_BLOCKS 6
-#endif
-constexpr int kPatBlocks = AMG_PAT_BLOCKS;  // resident blocks per SM the kernels are compiled for
+constexpr int kPatBlocks = 6;  // resident blocks per SM the kernels are compiled for
 
 // The table as the kernels hold it.  FP32 keeps an entry's value and offset
 // side by side, one 8-byte shared load per entry: two loads made the 27-point

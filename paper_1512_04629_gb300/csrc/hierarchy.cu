@@ -27,7 +27,6 @@ Hierarchy::~Hierarchy() {
     cudaGetDevice(&cur);
     if (cur == device && cudaDeviceSynchronize() == cudaSuccess) idle_release.enter();
     if (g_update) cudaGraphExecDestroy(g_update);
-    if (g_precond) cudaGraphExecDestroy(g_precond);
     if (graph_stream) cudaStreamDestroy(graph_stream);
     for (auto &p : pending) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto e : event_pool) cudaEventDestroy(e);

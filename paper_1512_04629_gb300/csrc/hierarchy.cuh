@@ -158,7 +158,7 @@ struct Hierarchy {
     std::vector<cudaEvent_t> event_pool;
 
     // CUDA graphs of the PCG iteration halves (captured per stream)
-    cudaGraphExec_t g_update = nullptr, g_precond = nullptr;
+    cudaGraphExec_t g_update = nullptr;
     cudaStream_t graph_stream = nullptr;
     bool graph_dirty = true;
     int version = 0;  // bumped whenever the cycle's buffers or operators change
