@@ -104,19 +104,30 @@ __device__ __forceinline__ void entries(int32_t e, const int32_t *__restrict__ c
 // acc += sum over the row's entries, in entry order, of a_ij * src_j[c0 ..]
 // (SCALE: times dinv_j, for x_j = dinv_j b_j that was never written); SUB:
 // subtracted, for residuals whose accumulator starts at b.  kAhead entries
-// at a time, the rest by halves.  In FP64 the rest is written as loops, which
-// the compiler leaves as branches: as plain conditions it predicates them,
-// and a predicated-off FMA holds the FP64 pipe like a real one -- in A p over
-// rows of five entries (4 + 1) the two absent ones took 501 us instead of 399
-// at 2D 2048^2, K = 8.  In FP32 conditions are the faster form (lognormal
-// 112^3, K = 32: 0.8% of the solve).
-template <typename VT, typename XT, int K, bool SCALE, bool SUB>
+// at a time, then the rest.  In FP64 the rest must be branches: as plain
+// conditions (entries<2>, entries<1>) the compiler predicates it, and a
+// predicated-off FMA holds the FP64 pipe like a real one -- in A p over rows of
+// five entries (4 + 1) the two absent ones took 501 us instead of 399 at 2D
+// 2048^2, K = 8.  A switch with all of the rest in flight (SWITCH, A p) and
+// loops of two and one (the FP64 cycle's passes, whose registers the switch
+// spills) compile to branches: lognormal 160^3, K = 64, FP32 cycle 485 ms with
+// loops in A p, 477 with the switch; 128^3, K = 32, FP64 250 with loops in the
+// passes, 254 with the switch, 259 with conditions.  In FP32 conditions are
+// the fastest form (lognormal 112^3, K = 32: by 0.8% of the solve).
+template <typename VT, typename XT, int K, bool SCALE, bool SUB, bool SWITCH = false>
 __device__ __forceinline__ void row_block_sum(int32_t p0, int32_t p1, const int32_t *__restrict__ ci,
                                               const VT *__restrict__ v, const XT *__restrict__ src,
                                               const XT *__restrict__ dinv, int c0, XT (&acc)[16 / sizeof(XT)]) {
     int32_t e = p0;
     for (; e + kAhead <= p1; e += kAhead) entries<kAhead, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
-    if constexpr (sizeof(XT) == 8) {
+    if constexpr (SWITCH) {
+        switch (p1 - e) {
+            case 3: entries<3, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc); break;
+            case 2: entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc); break;
+            case 1: entries<1, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc); break;
+            default: break;
+        }
+    } else if constexpr (sizeof(XT) == 8) {
 #pragma unroll 1
         for (; e + 2 <= p1; e += 2) entries<2, VT, XT, K, SCALE, SUB>(e, ci, v, src, dinv, c0, acc);
 #pragma unroll 1
@@ -438,7 +449,7 @@ ap_kernel(int32_t n, const int32_t *__restrict__ rp, const int32_t *__restrict__
         double acc[W] = {0.0, 0.0};
         const int64_t base = i * K + c0;
         if (RESID) vload(Bin + base, acc);
-        row_block_sum<double, double, K, false, RESID>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, Pin, nullptr, c0, acc);
+        row_block_sum<double, double, K, false, RESID, true>(__ldg(rp + i), __ldg(rp + i + 1), ci, v, Pin, nullptr, c0, acc);
         if (RESID) {
 #pragma unroll
             for (int w = 0; w < W; ++w) part[w] += acc[w] * acc[w];
